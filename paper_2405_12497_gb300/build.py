@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librabitq.so")
 BUILD_DIR = os.path.join(HERE, "_build")
 SOURCES = [
-    "api.cu", "api_predictor.cu", "kernels_gemm.cu", "kernels_build.cu", "kernels_search.cu",
+    "api.cu", "api_predictor.cu", "kernels_gemm.cu", "kernels_build.cu", "kernels_search.cu", "kernels_bucket.cu",
     "kernels_tc.cu", "kernels_mlp.cu", "noalloc.cu", "plan.cu", "shard.cu",
     "server.cu",
 ]

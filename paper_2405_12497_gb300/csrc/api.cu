@@ -67,6 +67,8 @@ void free_index_arrays(rabitq_index* X) {
   cudaFree(X->cn2);
   cudaFree(X->cnorm);
   cudaFree(X->cnorm_max);
+  cudaFree(X->rows8);
+  cudaFree(X->cent_rot);
 }
 
 int alloc_index_arrays(rabitq_index* X) {
@@ -90,6 +92,7 @@ int alloc_index_arrays(rabitq_index* X) {
   RBQ_CHECK(dev_alloc(&X->cn2, (size_t)X->K));
   RBQ_CHECK(dev_alloc(&X->cnorm, (size_t)X->K));
   RBQ_CHECK(dev_alloc(&X->cnorm_max, 1));
+  RBQ_CHECK(dev_alloc(&X->cent_rot, (size_t)X->K * ((X->d + 31) / 32 * 32)));
   return RABITQ_OK;
 }
 
@@ -257,6 +260,7 @@ int rabitq_build(const float* data, int64_t n, int32_t d, int32_t n_clusters, ui
     RBQ_CHECK(counting_sort(X->assign, n, n_clusters, X->perm, X->bucket_off, s));
     RBQ_CHECK(invert_perm(X->perm, n, X->inv_perm, s));
     RBQ_CHECK(gather_rows_f32(ddata, d, X->perm, n, d, X->data_b, s));
+    RBQ_CHECK(pack_rows(X, s));
     RBQ_CHECK(adist_b.alloc(sizeof(float) * n, s));
     RBQ_CHECK(gather_rows_f32(adist.as<float>(), 1, X->perm, n, 1, adist_b.as<float>(), s));
     RBQ_CHECK(sample_rotation_dev(seed, dpad, X->P64, X->P32, s));
@@ -845,6 +849,7 @@ int rabitq_index_load(const char* path, const rabitq_build_opts* opts, rabitq_in
       st = fail(RABITQ_ECUDA, "copy of P to the device failed");
     if (st == RABITQ_OK) st = pack_pt(X, nullptr);
   }
+  if (st == RABITQ_OK) st = pack_rows(X, nullptr);
   if (st == RABITQ_OK) st = max_bucket_size(X, nullptr);
   if (st != RABITQ_OK) {
     free_index_arrays(X);

@@ -49,6 +49,13 @@ struct rabitq_index {
   float* cn2 = nullptr;
   float* cnorm = nullptr;
   float* cnorm_max = nullptr;  // max ||c|| (one value)
+  // centroid rows for scattered reads by one lane each: K x 32-column lines
+  // (d rounded up, zeros), the four 32-byte sectors of a line rotated by the
+  // centroid's index (row_score_rot)
+  float* cent_rot = nullptr;
+  // 8-bit copy of the rows with its error bound, bucket order (pack_rows in
+  // kernels_bucket.cu; null when there was no memory for it)
+  uint8_t* rows8 = nullptr;
 };
 
 // Learned probe-count predictor (kernels_mlp.cu): MLP weights with BF16
@@ -187,6 +194,8 @@ struct ProbeScratch {
   // ascending: the key rounded up to a multiple of 128 | the centroid's index
   // among the 128 (0xffffffff past the last centroid)
   uint32_t* pool;
+  int* redo;        // 1 + M: count, queries left to the CTA selection
+  int* redo_mlp;    // 1 + M: count, queries with more than 64 learned probes
   int pool_n;       // kProbePool x (K / 128, rounded up to whole tiles of 256)
   size_t floats;    // total size
 };
@@ -228,6 +237,10 @@ struct SearchArgs {
   // captured) around the stages: distances | selection (+ MLP) | rotation |
   // fused scan, prune and re-rank. Single-chunk searches only.
   cudaEvent_t* stage_ev = nullptr;
+  // plans: a stream (and two events) for the query rotation, which runs beside
+  // the probe selection; null = everything in order on one stream
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
   // a batch too small to fill the GPU may split each query's probes over
   // several CTAs and merge them (identical results); off where scratch is fixed
   int allow_split = 1;
@@ -240,6 +253,9 @@ struct SearchArgs {
   // taken for batches that fill the GPU, while an explicit RABITQ_LAYOUT_WARP
   // request is taken for every batch
   int32_t tile_layout = 0;
+  // large batches may take the bucket-major scan (kernels_bucket.cu); off where
+  // the scratch is fixed
+  int allow_bucket = 1;
   // bulk-copy staging of the CTA layout's scan rounds (RABITQ_STAGING_*;
   // AUTO resolves to the tuned or default choice)
   int32_t stage = 0;
@@ -273,6 +289,14 @@ int search_enqueue_carved(const SearchArgs& a, unsigned char* scratch, size_t sc
                           int64_t grid, int64_t cap, cudaStream_t s);
 // scratch bytes for nq_max queries in one chunk with a.cand_cap candidates per CTA
 size_t carved_bytes(const SearchArgs& a, int64_t grid, int64_t nq_max);
+// ---- bucket-major scan of large batches (kernels_bucket.cu)
+struct FusedParams;
+// whether a batch of nq queries takes it (an AUTO layout, many pairs per bucket)
+bool bucket_applies(const SearchArgs& a, int64_t nq);
+size_t bucket_bytes(const SearchArgs& a, int64_t nq);
+int pack_rows(rabitq_index* X, cudaStream_t s);
+int bucket_search(const SearchArgs& a, const FusedParams& P, unsigned char* scratch,
+                  void (*fn)(FusedParams), unsigned grid, size_t fn_smem, cudaStream_t s);
 // CTAs of the fused kernel at full residency for these search parameters
 int fused_grid(const SearchArgs& a, int* grid_out);
 
@@ -294,9 +318,19 @@ int mlp_adam(float* master, float* work, const float* g, float* m1, float* m2, f
 // navail = min(64, K) valid entries)
 int mlp_features(const float* sel_dist, int64_t ld, int64_t nq, int navail, float s0, float* X,
                  cudaStream_t s);
-// fused inference: features, MLP and probe counts in one kernel
+// fused inference: features, MLP and probe counts in one kernel, and with
+// lists.out_ids also the probe lists of the queries that need at most navail
+// buckets (their ids: sel_ids, rows of ld), the others in redo
+struct MlpLists {
+  const int32_t* sel_ids = nullptr;
+  int32_t* out_ids = nullptr;  // nq x ldo
+  float* out_dist = nullptr;
+  int64_t ldo = 0;
+  int* redo = nullptr;         // count (zeroed by the caller), then the queries
+};
 int mlp_infer(const rabitq_predictor* pr, const float* sel_dist, int64_t ld, int64_t nq,
-              int navail, int32_t* nprobe_out, float* feat, float* y, cudaStream_t s);
+              int navail, int32_t* nprobe_out, float* feat, float* y, cudaStream_t s,
+              const MlpLists& lists = MlpLists());
 // in = out allowed; packed (BF16) may be null
 int mlp_round(const float* in, float* out, void* packed, int n, cudaStream_t s);
 // neighbours a label must cover: ceil(target k), with a tolerance of 1e-6 k

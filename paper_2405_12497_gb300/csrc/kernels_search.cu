@@ -25,12 +25,12 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "query_common.cuh"
 #include "tc_util.cuh"
 
 namespace rbq {
 namespace {
 
-constexpr int kThreads = 256;
 
 // ------------------------------------------------------------ selection
 // Top-nsel of K scores score(c) by (score, id): radix select of the nsel-th
@@ -117,777 +117,6 @@ __device__ void select_row(F score, int K, int nsel, int nprobe, int sort_n,
 }
 
 
-// ------------------------------------------------------ fused query kernel
-// Shared state of the block radix select.
-struct SelState {
-  int hist[256];
-  int bin, rem, tie_taken;
-  int warp_cnt[kThreads / 32];
-  unsigned long long wmin[kThreads / 32], wmax[kThreads / 32];
-};
-
-struct FusedParams {
-  const float* queries;     // nq x d
-  const float* rq;          // nq x dpad
-  const int32_t* probe_ids; // nq x nprobe
-  const float* probe_dist;  // nq x nprobe: centroid scores, the estimator's additive term
-  const float* probe_nq2;   // nq x nprobe ||q_r - c||^2 (IP metric), null = probe_dist
-  const int32_t* nprobe_q;  // nq or null
-  const float* ptc;         // K x dpad
-  const uint64_t* codes;    // n x W (bucket order)
-  const float4* factors;    // n (bucket order)
-  const float* data_b;      // n x d (bucket order)
-  const int32_t* perm;      // n: position -> id
-  const int32_t* inv_perm;  // n: id -> position
-  const int32_t* bucket_off;
-  int64_t nq, q_offset;
-  int d, dpad, W, bq, k, m, nprobe, pch, cu, ce, ct;
-  float eps0;
-  uint64_t seed;
-  int cand_cap;
-  int metric;               // 0: squared distance; 1: inner product (score -<o_r, q_r>)
-  int4* cand;               // gridDim.x x cand_cap: {pos, LB, estimate, -}
-  int64_t* out_ids;
-  float* out_dist;
-  int* err;
-  rabitq_trace tr;
-  // query scheduling: CTAs take the next query from *next (zeroed before the
-  // launch) in the order `order` (null = ascending); next == null = static
-  // striding by gridDim.x
-  const int32_t* order;
-  int* next;
-  int scap;  // shared-memory capacity for the tail's candidate list (0 = none)
-  // Split mode (split > 1, for batches too small to fill the GPU): work item
-  // i scans probe slice i % split of query i / split into candidate region i
-  // and writes the slice's k smallest upper-bound keys to ub_out[i k ...] and
-  // {keys written, candidates} to slice_cnt[2 i ...]; split_merge_kernel
-  // then finishes each query from its slices. cand2: one merged-list region
-  // of cand_cap entries per query.
-  int split;
-  uint32_t* ub_out;
-  int* slice_cnt;
-  int4* cand2;
-  // Warp-per-query kernel: candidate region of capw entries per warp; a
-  // query whose list outgrows it goes to redo[*redo_cnt++]. The CTA kernel
-  // redoing them reads its query count from *nq_dev when that is set.
-  int4* candw;
-  int capw;
-  int32_t* redo;
-  int* redo_cnt;
-  const int* nq_dev;
-};
-
-struct FusedSmem {
-  uint64_t* planes;  // pch x bq x W
-  float4* pmeta;     // pch: A, B, E, nq2
-  int* psum;         // pch
-  int* pbeg;         // pch
-  int* pref;         // pch + 1
-  float* qv;         // d
-  SelState* sel;     // radix-select scratch
-  uint32_t* ubk;     // cu: upper-bound keys
-  unsigned long long* estk;  // ce: the pilot list, (id << 32) | position
-  unsigned long long* topk;  // ct: (exact distance key << 32) | id
-  int4* scand;               // scap: the candidate list staged for the tail
-};
-
-__host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-
-__host__ __device__ inline size_t fused_smem_bytes(int pch, int bq, int W, int d, int cu, int ce,
-                                                   int ct, int nwarps,
-                                                   size_t* off /* 10 entries or null */,
-                                                   int scap = 0) {
-  size_t o = 0, offs[10];
-  (void)nwarps;
-  offs[0] = o; o = align_up(o + sizeof(uint64_t) * pch * bq * W, 16);
-  offs[1] = o; o = align_up(o + sizeof(float4) * pch, 16);
-  offs[2] = o; o = align_up(o + sizeof(int) * pch, 16);
-  offs[3] = o; o = align_up(o + sizeof(int) * pch, 16);
-  offs[4] = o; o = align_up(o + sizeof(int) * (pch + 1), 16);
-  offs[5] = o; o = align_up(o + sizeof(float) * d, 16);
-  offs[6] = o; o = align_up(o + sizeof(uint32_t) * cu, 16);
-  offs[7] = o; o = align_up(o + sizeof(unsigned long long) * ce, 16);
-  offs[8] = o; o = align_up(o + sizeof(unsigned long long) * ct, 16);
-  offs[9] = o; o = align_up(o + sizeof(int4) * scap, 16);
-  if (off)
-    for (int i = 0; i < 10; ++i) off[i] = offs[i];
-  return o;
-}
-
-// Randomized B_q-bit quantization of q' for one probed cluster with one warp
-// (§3.3.1): qd = rq - P^T c, v_l = min qd, v_r = max qd, Delta = (v_r -
-// v_l)/(2^B_q - 1), q_u[k] = min(floor((qd[k] - v_l)/Delta + u_k), 2^B_q - 1)
-// with u_k from Philox(seed; k/4, query, cluster, 3). Lane l holds elements
-// k = 128 i + 4 l + r (r = 0..3), so the four u_k of one Philox call belong to
-// one lane; emit(i, k0, qu) receives them block by block (warp-uniform).
-// Returns sum(q_u) in every lane; writes v_l and Delta.
-template <class Emit>
-__device__ __forceinline__ int quant_core(const float* rq, const float* pc, int dpad, int bq,
-                                          uint64_t seed, uint64_t gq, int c, float* vl_out,
-                                          float* delta_out, Emit emit) {
-  const int lane = threadIdx.x & 31;
-  const int nblk = (dpad + 127) >> 7;
-  float vl = __int_as_float(0x7f800000), vr = __int_as_float(0xff800000);
-  for (int kk = lane; kk < dpad; kk += 32) {
-    const float v = __fsub_rn(rq[kk], pc[kk]);
-    vl = fminf(vl, v);
-    vr = fmaxf(vr, v);
-  }
-  vl = warp_min_f(vl);
-  vr = warp_max_f(vr);
-  const int qmax = (1 << bq) - 1;
-  const float delta = __fdiv_rn(__fsub_rn(vr, vl), (float)qmax);
-  int sum = 0;
-  for (int i = 0; i < nblk; ++i) {
-    const int k0 = 128 * i + 4 * lane;
-    int qu[4] = {0, 0, 0, 0};
-    if (delta > 0.0f && k0 < dpad) {
-      float qd[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) qd[r] = (k0 + r < dpad) ? __fsub_rn(rq[k0 + r], pc[k0 + r]) : 0.0f;
-      const U4 w = philox4x32_10(seed, (uint32_t)(k0 >> 2), (uint32_t)gq, (uint32_t)c, kTagQuant);
-      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        if (k0 + r < dpad) {
-          const float u = __fmul_rn(__uint2float_rn(ws[r] >> 8), 0x1.0p-24f);
-          const float x = __fdiv_rn(__fsub_rn(qd[r], vl), delta);
-          const int v = __float2int_rd(__fadd_rn(x, u));
-          qu[r] = v > qmax ? qmax : v;
-        }
-      }
-    }
-    sum += qu[0] + qu[1] + qu[2] + qu[3];
-    emit(i, k0, qu);
-  }
-  *vl_out = vl;
-  *delta_out = delta;
-  return warp_sum_i(sum);
-}
-
-// Per-(query, cluster) constants of the estimator: A = Delta/sqrt(D'),
-// B = v_l/sqrt(D'), E = ||q_r - c|| 2 eps0/sqrt(D'-1) and the additive term
-// add: ||q_r - c||^2 for distances, -<q_r, c> for inner products (§6).
-__device__ __forceinline__ float4 quant_meta(float delta, float vl, float nq2, float add,
-                                             float eps0, int dpad) {
-  const float sqd = __fsqrt_rn((float)dpad);
-  const float keps = __fdiv_rn(__fmul_rn(2.0f, eps0), __fsqrt_rn((float)(dpad - 1)));
-  const float n_q = __fsqrt_rn(nq2);
-  return make_float4(__fdiv_rn(delta, sqd), __fdiv_rn(vl, sqd), __fmul_rn(n_q, keps), add);
-}
-
-// Quantize for the popcount scan: B_q bit-planes of q_u into shared memory.
-__device__ __forceinline__ void quantize_probe(const FusedParams& P, const FusedSmem& S, int64_t q,
-                                               int j, int jg, int c, float nq2, float add) {
-  const int lane = threadIdx.x & 31;
-  const int dpad = P.dpad, W = P.W, bq = P.bq;
-  uint64_t* planes = S.planes + (size_t)j * bq * W;
-  float vl, delta;
-  const int sum = quant_core(
-      P.rq + q * dpad, P.ptc + (int64_t)c * dpad, dpad, bq, P.seed, (uint64_t)(P.q_offset + q), c,
-      &vl, &delta, [&](int i, int, const int* qu) {
-        // the nibble of lane l sits at bits 4l..4l+3 of the 128-bit block
-        for (int b = 0; b < bq; ++b) {
-          const uint32_t nib = ((qu[0] >> b) & 1) | (((qu[1] >> b) & 1) << 1) |
-                               (((qu[2] >> b) & 1) << 2) | (((qu[3] >> b) & 1) << 3);
-          const uint32_t part = nib << (4 * (lane & 7));
-          const uint32_t q0 = __reduce_or_sync(kFull, lane < 8 ? part : 0u);
-          const uint32_t q1 = __reduce_or_sync(kFull, (lane >= 8 && lane < 16) ? part : 0u);
-          const uint32_t q2 = __reduce_or_sync(kFull, (lane >= 16 && lane < 24) ? part : 0u);
-          const uint32_t q3 = __reduce_or_sync(kFull, lane >= 24 ? part : 0u);
-          if (lane == 0) {
-            const int w0 = 2 * i;
-            if (w0 < W) planes[b * W + w0] = ((uint64_t)q1 << 32) | q0;
-            if (w0 + 1 < W) planes[b * W + w0 + 1] = ((uint64_t)q3 << 32) | q2;
-          }
-        }
-      });
-  if (lane == 0) {
-    const float4 m = quant_meta(delta, vl, nq2, add, P.eps0, dpad);
-    S.pmeta[j] = m;
-    S.psum[j] = sum;
-    S.pbeg[j] = P.bucket_off[c];
-    S.pref[j + 1] = P.bucket_off[c + 1] - P.bucket_off[c];  // length; prefix-summed later
-    if (P.tr.sum_qu) P.tr.sum_qu[q * P.nprobe + jg] = sum;
-    if (P.tr.meta) {
-      float* tm = P.tr.meta + (q * P.nprobe + jg) * 4;
-      tm[0] = m.x; tm[1] = m.y; tm[2] = m.z; tm[3] = m.w;
-    }
-  }
-  __syncwarp();
-  if (P.tr.planes) {
-    uint64_t* tp = P.tr.planes + (q * P.nprobe + jg) * (int64_t)bq * W;
-    for (int t = lane; t < bq * W; t += 32) tp[t] = planes[t];
-  }
-}
-
-// Warp-aggregated slot reservation: lanes with `want` get consecutive slots
-// from one atomicAdd per warp (shared-memory counters are hot).
-__device__ __forceinline__ int warp_reserve(bool want, int* counter) {
-  const unsigned m = __ballot_sync(kFull, want);
-  if (m == 0) return -1;
-  const int lane = threadIdx.x & 31;
-  const int leader = __ffs(m) - 1;
-  int base = 0;
-  if (lane == leader) base = atomicAdd(counter, __popc(m));
-  base = __shfl_sync(kFull, base, leader);
-  return want ? base + __popc(m & ((1u << lane) - 1u)) : -1;
-}
-
-
-// ---------------------------------------------------------- block select
-// The want-th smallest (1-based, want <= n) of the n keys a[0..n) by an
-// MSD radix select, 8 bits per pass; histogram updates are aggregated per
-// warp by digit. On return st.rem = how many keys equal to the result are
-// among the `want` smallest. Whole block; synchronized on return.
-template <class K, class F>
-__device__ K block_select_f(int n, int want, SelState& st, F keyf) {
-  constexpr int NB = (int)sizeof(K) * 8;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // The leading bits where the smallest and the largest key agree are common
-  // to every key and need no histogram pass: one min/max pass finds them.
-  K kmin = ~(K)0, kmax = 0;
-  for (int i = tid; i < n; i += blockDim.x) {
-    const K key = keyf(i);
-    kmin = key < kmin ? key : kmin;
-    kmax = key > kmax ? key : kmax;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const K a = __shfl_xor_sync(kFull, kmin, o), b = __shfl_xor_sync(kFull, kmax, o);
-    kmin = a < kmin ? a : kmin;
-    kmax = b > kmax ? b : kmax;
-  }
-  if (lane == 0) {
-    st.wmin[wid] = kmin;
-    st.wmax[wid] = kmax;
-  }
-  __syncthreads();
-  kmin = ~(K)0;
-  kmax = 0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-    kmin = (K)st.wmin[w] < kmin ? (K)st.wmin[w] : kmin;
-    kmax = (K)st.wmax[w] > kmax ? (K)st.wmax[w] : kmax;
-  }
-  if (kmin == kmax) {  // all keys equal: the answer, with every key a tie
-    __syncthreads();
-    if (tid == 0) {
-      st.bin = (int)(kmin & 255);
-      st.hist[st.bin] = n;
-      st.rem = want;
-    }
-    __syncthreads();
-    return kmin;
-  }
-  const K diff = kmin ^ kmax;
-  const int top = NB - 1 - (sizeof(K) == 8 ? __clzll((long long)diff) : __clz((int)diff));
-  const int start = (top / 8) * 8;  // the byte holding the highest differing bit
-  K mask = start + 8 >= NB ? (K)0 : ~(((K)1 << (start + 8)) - 1);
-  K prefix = kmin & mask;
-  int rem = want;
-  for (int shift = start; shift >= 0; shift -= 8) {
-    for (int i = tid; i < 256; i += blockDim.x) st.hist[i] = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < n; b0 += blockDim.x) {
-      const int i = b0 + tid;
-      K key = 0;
-      bool v = false;
-      if (i < n) {
-        key = keyf(i);
-        v = (key & mask) == prefix;
-      }
-      const int dig = v ? (int)((key >> shift) & 255) : 256 + lane;
-      const unsigned grp = __match_any_sync(kFull, dig);
-      if (v && lane == __ffs(grp) - 1) atomicAdd(&st.hist[dig], __popc(grp));
-    }
-    __syncthreads();
-    if (tid < 32) {
-      int c[8], sum = 0;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        c[u] = st.hist[lane * 8 + u];
-        sum += c[u];
-      }
-      int incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const unsigned hit = __ballot_sync(kFull, incl >= rem);
-      if (lane == __ffs(hit) - 1) {
-        int cum = incl - sum;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (cum + c[u] >= rem) {
-            st.bin = lane * 8 + u;
-            st.rem = rem - cum;
-            break;
-          }
-          cum += c[u];
-        }
-      }
-    }
-    __syncthreads();
-    prefix |= (K)st.bin << shift;
-    mask |= (K)255 << shift;
-    rem = st.rem;
-    __syncthreads();
-  }
-  return prefix;
-}
-
-template <class K>
-__device__ K block_select(const K* a, int n, int want, SelState& st) {
-  return block_select_f<K>(n, want, st, [a](int i) { return a[i]; });
-}
-
-// The want-th smallest (1-based, want <= n) of n 32-bit keys: one histogram
-// of kHistBins equal-width bins over [min, max] (bin = (key - min) kHistBins
-// / (max - min + 1): monotone in the key, so the bins order the keys), then
-// an exact selection among the keys of the boundary bin, collected into coll
-// (ranked directly when they fit one per thread). rem = how many keys equal
-// to the result are among the want smallest, eq = how many keys equal it in
-// all. hist: kHistBins ints; coll: coll_cap keys. Falls back to the radix
-// select when the boundary bin does not fit coll. Whole block (kThreads
-// threads); synchronized on return.
-constexpr int kHistBins = 1024;
-template <class F>
-__device__ uint32_t hist_select(int n, int want, SelState& st, int* hist, uint32_t* coll,
-                                int coll_cap, int& rem, int& eq, F keyf) {
-  static_assert(kHistBins == 4 * kThreads, "four bins per thread");
-  __shared__ int s_hs[5];  // boundary bin, keys below it, fill, rem, eq
-  __shared__ uint32_t s_T;
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-  uint32_t kmin = 0xffffffffu, kmax = 0u;
-  for (int i = tid; i < n; i += blockDim.x) {
-    const uint32_t key = keyf(i);
-    kmin = key < kmin ? key : kmin;
-    kmax = key > kmax ? key : kmax;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint32_t a = __shfl_xor_sync(kFull, kmin, o), b = __shfl_xor_sync(kFull, kmax, o);
-    kmin = a < kmin ? a : kmin;
-    kmax = b > kmax ? b : kmax;
-  }
-  if (lane == 0) {
-    st.wmin[wid] = kmin;
-    st.wmax[wid] = kmax;
-  }
-  __syncthreads();
-  kmin = 0xffffffffu;
-  kmax = 0u;
-  for (int w = 0; w < nw; ++w) {
-    kmin = (uint32_t)st.wmin[w] < kmin ? (uint32_t)st.wmin[w] : kmin;
-    kmax = (uint32_t)st.wmax[w] > kmax ? (uint32_t)st.wmax[w] : kmax;
-  }
-  if (kmin == kmax) {  // all keys equal
-    rem = want;
-    eq = n;
-    __syncthreads();
-    return kmin;
-  }
-  const uint64_t span = (uint64_t)(kmax - kmin) + 1u;
-  auto bin_of = [kmin, span](uint32_t key) {
-    return (int)(((uint64_t)(key - kmin) * (uint64_t)kHistBins) / span);
-  };
-  for (int i = tid; i < kHistBins; i += blockDim.x) hist[i] = 0;
-  __syncthreads();
-  for (int i = tid; i < n; i += blockDim.x) atomicAdd(&hist[bin_of(keyf(i))], 1);
-  __syncthreads();
-  // the bin holding the want-th key: four bins per thread, block prefix sum
-  int c[4], sum = 0;
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    c[u] = hist[4 * tid + u];
-    sum += c[u];
-  }
-  int incl = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) st.warp_cnt[wid] = incl;
-  __syncthreads();
-  for (int w = 0; w < wid; ++w) incl += st.warp_cnt[w];
-  const int excl = incl - sum;
-  if (excl < want && incl >= want) {  // exactly one thread
-    int cum = excl;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (cum + c[u] >= want) {
-        s_hs[0] = 4 * tid + u;
-        s_hs[1] = cum;
-        break;
-      }
-      cum += c[u];
-    }
-  }
-  if (tid == 0) s_hs[2] = 0;
-  __syncthreads();
-  const int B = s_hs[0], below = s_hs[1], nB = hist[B], want_b = want - below;
-  uint32_t T;
-  if (nB <= coll_cap) {
-    for (int b0 = 0; b0 < n; b0 += blockDim.x) {
-      const int i = b0 + tid;
-      uint32_t key = 0u;
-      bool in = false;
-      if (i < n) {
-        key = keyf(i);
-        in = bin_of(key) == B;
-      }
-      const int slot = warp_reserve(in, &s_hs[2]);
-      if (in) coll[slot] = key;
-    }
-    __syncthreads();
-    if (nB <= (int)blockDim.x) {  // rank each key of the bin against the others
-      if (tid < nB) {
-        const uint32_t mine = coll[tid];
-        int lt = 0, le = 0;
-        for (int j = 0; j < nB; ++j) {
-          const uint32_t v = coll[j];
-          lt += v < mine ? 1 : 0;
-          le += v <= mine ? 1 : 0;
-        }
-        if (lt < want_b && want_b <= le) {  // the threads holding the result
-          s_T = mine;
-          s_hs[3] = want_b - lt;
-          s_hs[4] = le - lt;
-        }
-      }
-      __syncthreads();
-      T = s_T;
-      rem = s_hs[3];
-      eq = s_hs[4];
-    } else {
-      T = block_select_f<uint32_t>(nB, want_b, st, [coll](int i) { return coll[i]; });
-      rem = st.rem;
-      eq = st.hist[st.bin];
-    }
-  } else {
-    T = block_select_f<uint32_t>(n, want, st, keyf);
-    rem = st.rem;
-    eq = st.hist[st.bin];
-  }
-  __syncthreads();
-  return T;
-}
-
-// In place, keep the keys below T and `ties` of the keys equal to T; returns
-// the new count (whole block; synchronized on return).
-template <class K>
-__device__ int block_keep_below(K* a, int n, K T, int ties, SelState& st) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  if (tid == 0) st.tie_taken = 0;
-  __syncthreads();
-  int out = 0;
-  for (int b0 = 0; b0 < n; b0 += blockDim.x) {
-    const int i = b0 + tid;
-    K key = 0;
-    bool keep = false;
-    if (i < n) {
-      key = a[i];
-      keep = key < T || (key == T && atomicAdd(&st.tie_taken, 1) < ties);
-    }
-    const unsigned bal = __ballot_sync(kFull, keep);
-    if (lane == 0) st.warp_cnt[wid] = __popc(bal);
-    __syncthreads();
-    int before = out, tot = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      if (w < wid) before += st.warp_cnt[w];
-      tot += st.warp_cnt[w];
-    }
-    if (keep) a[before + __popc(bal & ((1u << lane) - 1u))] = key;
-    out += tot;
-    __syncthreads();
-  }
-  return out;
-}
-
-// Keep the `keep` smallest of the *cnt keys (no order); returns the
-// keep-th smallest key (or ~0 if there are fewer than keep keys).
-template <class K>
-__device__ K select_keep(K* a, int* cnt, int keep, SelState& st) {
-  const int n = *cnt;
-  if (n < keep) {
-    __syncthreads();
-    return ~(K)0;
-  }
-  const K T = block_select<K>(a, n, keep, st);
-  const int kept = block_keep_below<K>(a, n, T, st.rem, st);
-  if (threadIdx.x == 0) *cnt = kept;
-  __syncthreads();
-  return T;
-}
-
-// select_keep for 32-bit keys by the histogram select (hist, coll: shared
-// memory the caller has free at this point).
-__device__ uint32_t select_keep_h(uint32_t* a, int* cnt, int keep, SelState& st, int* hist,
-                                  uint32_t* coll, int coll_cap) {
-  const int n = *cnt;
-  if (n < keep) {
-    __syncthreads();
-    return 0xffffffffu;
-  }
-  int rem = 0, eq = 0;
-  const uint32_t T =
-      hist_select(n, keep, st, hist, coll, coll_cap, rem, eq, [a](int i) { return a[i]; });
-  const int kept = block_keep_below<uint32_t>(a, n, T, rem, st);
-  if (threadIdx.x == 0) *cnt = kept;
-  __syncthreads();
-  return T;
-}
-
-// Keep the `keep` smallest of the *cnt distinct (distance key << 32 | id)
-// keys of a: a 32-bit select on the distance half (by the histogram select
-// when hist/coll are given, else the radix select), then -- only when more
-// keys share the boundary distance than are kept -- one on the id half of
-// those. Returns the keep-th smallest key (~0 if there are fewer than keep).
-// Whole block; synchronized on return.
-__device__ unsigned long long select_keep_dk(unsigned long long* a, int* cnt, int keep,
-                                             SelState& st, int* hist = nullptr,
-                                             uint32_t* coll = nullptr, int coll_cap = 0) {
-  const int n = *cnt;
-  if (n < keep) {
-    __syncthreads();
-    return ~0ull;
-  }
-  uint32_t Td;
-  int ties = 0, eqn = 0;
-  if (hist) {
-    Td = hist_select(n, keep, st, hist, coll, coll_cap, ties, eqn,
-                     [a](int i) { return (uint32_t)(a[i] >> 32); });
-  } else {
-    Td = block_select_f<uint32_t>(n, keep, st, [a](int i) { return (uint32_t)(a[i] >> 32); });
-    ties = st.rem;
-    eqn = st.hist[st.bin];
-  }
-  uint32_t Tid = 0xffffffffu;
-  if (eqn > ties)
-    Tid = block_select_f<uint32_t>(n, ties, st, [a, Td](int i) {
-      return (uint32_t)(a[i] >> 32) == Td ? (uint32_t)(a[i] & 0xffffffffu) : 0xffffffffu;
-    });
-  unsigned long long T = ((unsigned long long)Td << 32) | Tid;
-  if (Tid == 0xffffffffu) {  // every key at the boundary distance is kept
-    T = ((unsigned long long)Td << 32) | 0xffffffffu;
-  }
-  const int kept = block_keep_below<unsigned long long>(a, n, T, 1, st);
-  if (threadIdx.x == 0) *cnt = kept;
-  __syncthreads();
-  if (Tid == 0xffffffffu) {
-    // the keep-th smallest key itself: the largest kept key
-    __shared__ unsigned long long s_max;
-    if (threadIdx.x == 0) s_max = 0;
-    __syncthreads();
-    unsigned long long mx = 0;
-    for (int i = threadIdx.x; i < kept; i += blockDim.x) mx = a[i] > mx ? a[i] : mx;
-    atomicMax(&s_max, mx);
-    __syncthreads();
-    T = s_max;
-    __syncthreads();
-  }
-  return T;
-}
-
-// Sort the first pow2(keep) slots of a shared key buffer holding *cnt <=
-// keep keys (padded with the maximum key). Whole block; synchronized on return.
-__device__ __forceinline__ void sort_kept_u64(unsigned long long* a, int cnt, int keep) {
-  int n = 1;
-  while (n < keep) n <<= 1;
-  for (int i = cnt + threadIdx.x; i < n; i += blockDim.x) a[i] = ~0ull;
-  __syncthreads();
-  block_bitonic_sort_u64(a, n);
-  __syncthreads();
-}
-
-// In-place, order-keeping compaction of the candidate list with predicate f:
-// blocks of kCompactU x blockDim entries (kCompactU loads in flight per
-// thread, two barriers per block); every read of a block precedes its
-// writes, which land below the block's end. scratch: kCompactU x
-// (blockDim / 32) ints. (Two entries per thread: four cost the fused kernel
-// register spills that outweighed the fewer barriers.)
-constexpr int kCompactU = 2;
-template <class F>
-__device__ __forceinline__ void compact_cand(int4* cand, int* cnt, int cap, int* scratch, F keep_f) {
-  const int n = min(*cnt, cap);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const unsigned below = (1u << lane) - 1u;
-  int out = 0;
-  __syncthreads();
-  for (int b = 0; b < n; b += kCompactU * blockDim.x) {
-    int4 e[kCompactU];
-    bool keep[kCompactU];
-#pragma unroll
-    for (int u = 0; u < kCompactU; ++u) {
-      const int i = b + u * blockDim.x + threadIdx.x;
-      e[u] = make_int4(0, 0, 0, 0);
-      keep[u] = false;
-      if (i < n) {
-        e[u] = cand[i];
-        keep[u] = keep_f(e[u]);
-      }
-    }
-    unsigned bal[kCompactU];
-#pragma unroll
-    for (int u = 0; u < kCompactU; ++u) {
-      bal[u] = __ballot_sync(kFull, keep[u]);
-      if (lane == 0) scratch[u * nw + wid] = __popc(bal[u]);
-    }
-    __syncthreads();
-    // entry (u, thread) follows every kept entry of sub-blocks < u and of
-    // the warps before it in sub-block u
-#pragma unroll
-    for (int u = 0; u < kCompactU; ++u) {
-      int before = out, tot = 0;
-      for (int w = 0; w < nw; ++w) {
-        const int c = scratch[u * nw + w];
-        if (w < wid) before += c;
-        tot += c;
-      }
-      if (keep[u]) cand[before + __popc(bal[u] & below)] = e[u];
-      out += tot;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *cnt = out;
-  __syncthreads();
-}
-
-// One term of the canonical exact score: squared distance, fold of
-// (q - x)^2; inner product, fold of q x (negated at the end).
-template <bool IP>
-__device__ __forceinline__ float score_step(float acc, float q, float x) {
-  if (IP) return __fmaf_rn(q, x, acc);
-  const float t = __fsub_rn(q, x);
-  return __fmaf_rn(t, t, acc);
-}
-
-// Canonical exact score of row x against the query qv (shared memory), in
-// ascending dimension order: ||q - x||^2, or -<q, x> for inner products.
-// 32-byte loads, four in flight, when d is a multiple of 8 (rows, in
-// cudaMalloc'ed arrays, then start on 32-byte boundaries); 16-byte loads,
-// eight in flight, when d is a multiple of 4.
-template <bool IP>
-__device__ __forceinline__ float row_score(const float* __restrict__ x, const float* qv, int d) {
-  float acc = 0.0f;
-  if ((d & 7) == 0) {
-    // (qv: 16-byte aligned shared memory, read as float4)
-    const float4* q4 = reinterpret_cast<const float4*>(qv);
-    auto fold8 = [&](const unsigned long long (&v)[4], int c) {
-      const float4 qa = q4[c >> 2], qb = q4[(c >> 2) + 1];
-      const float qq[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        acc = score_step<IP>(acc, qq[e], __int_as_float((int)(uint32_t)(v[e >> 1] >> (32 * (e & 1)))));
-    };
-    int c = 0;
-    for (; c + 32 <= d; c += 32) {
-      unsigned long long v[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];"
-                     : "=l"(v[u][0]), "=l"(v[u][1]), "=l"(v[u][2]), "=l"(v[u][3])
-                     : "l"(x + c + 8 * u));
-#pragma unroll
-      for (int u = 0; u < 4; ++u) fold8(v[u], c + 8 * u);
-    }
-    for (; c < d; c += 8) {
-      unsigned long long v[4];
-      asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];"
-                   : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
-                   : "l"(x + c));
-      fold8(v, c);
-    }
-  } else if ((d & 3) == 0) {
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    const float4* q4 = reinterpret_cast<const float4*>(qv);
-    int c = 0;
-    for (; c + 8 <= (d >> 2); c += 8) {
-      float4 v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = __ldg(x4 + c + u);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float4 qq = q4[c + u];
-        acc = score_step<IP>(acc, qq.x, v[u].x);
-        acc = score_step<IP>(acc, qq.y, v[u].y);
-        acc = score_step<IP>(acc, qq.z, v[u].z);
-        acc = score_step<IP>(acc, qq.w, v[u].w);
-      }
-    }
-    for (; c < (d >> 2); ++c) {
-      const float4 vv = __ldg(x4 + c), qq = q4[c];
-      acc = score_step<IP>(acc, qq.x, vv.x);
-      acc = score_step<IP>(acc, qq.y, vv.y);
-      acc = score_step<IP>(acc, qq.z, vv.z);
-      acc = score_step<IP>(acc, qq.w, vv.w);
-    }
-  } else {
-    for (int dd = 0; dd < d; ++dd) acc = score_step<IP>(acc, qv[dd], __ldg(x + dd));
-  }
-  return IP ? -acc : acc;
-}
-
-// Exact scores of a list of rows: each lane streams its own row (a warp has
-// 256 rows' worth of loads outstanding) and folds it in ascending dimension
-// order. Keys (score, id) go to the top-k buffer.
-// SRC 0: the pilot (ids in S.estk); SRC 1: the candidate list (positions).
-// kmax: keys above it cannot enter the result and are not kept (the rest
-// of the re-rank set, once the pilot's k smallest keys are known).
-template <int SRC>
-__device__ void rerank_rows(const FusedParams& P, const FusedSmem& S, int64_t q, int count,
-                            const int4* cand, int* top_cnt, int* surv_cnt,
-                            unsigned long long kmax = ~0ull) {
-  const int d = P.d;
-  // Ask L2 for the rows of the first two rounds (no registers held, no
-  // waiting): their loads then find most rows in L2 instead of waiting on
-  // DRAM four loads at a time. (Asking for a whole set of thousands of rows
-  // at once, or two rounds ahead every round, measured slower.)
-  const int row_bytes = d * (int)sizeof(float);
-  for (int i = threadIdx.x; i < min(count, 2 * (int)blockDim.x); i += blockDim.x) {
-    const int pos = SRC == 0 ? (int)(S.estk[i] & 0xffffffffu) : (cand[i].x & 0x7fffffff);
-    const char* x = reinterpret_cast<const char*>(P.data_b + (int64_t)pos * d);
-    for (int o = 0; o < row_bytes; o += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + o));
-  }
-  for (int r0 = 0; r0 < count; r0 += blockDim.x) {
-    const int i = r0 + threadIdx.x;
-    const bool valid = i < count;
-    int pos = 0, id = 0;
-    if (valid) {
-      if (SRC == 0) {
-        const unsigned long long e = S.estk[i];
-        id = (int)(e >> 32);
-        pos = (int)(e & 0xffffffffu);
-      } else {
-        pos = cand[i].x & 0x7fffffff;
-        id = P.perm[pos];
-      }
-    }
-    float acc = 0.0f;
-    if (valid) {
-      const float* x = P.data_b + (int64_t)pos * d;
-      acc = P.metric ? row_score<true>(x, S.qv, d) : row_score<false>(x, S.qv, d);
-    }
-    const unsigned long long key = ((unsigned long long)float_key(acc) << 32) | (uint32_t)id;
-    const bool take = valid && key <= kmax;
-    const int slot = warp_reserve(take, top_cnt);
-    if (take) S.topk[slot] = key;
-    if (valid) {
-      const int si = i + (SRC == 0 ? 0 : *surv_cnt);
-      if (P.tr.surv_ids && si < P.tr.surv_cap) P.tr.surv_ids[q * P.tr.surv_cap + si] = id;
-    }
-    __syncthreads();
-    const int tc = *top_cnt;  // read between barriers (see the scan's upkeep)
-    __syncthreads();
-    if (tc > P.ct - (int)blockDim.x) select_keep_dk(S.topk, top_cnt, P.k, *S.sel);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) *surv_cnt += count;
-  __syncthreads();
-}
-
 // ------------------------------------------------------------ probe selection
 // The nsel nearest centroids of each query (§4's probe; for inner products
 // the largest <q_r, c>), exactly as a full canonical scan would rank them,
@@ -929,37 +158,31 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     const uint32_t* __restrict__ kmax_q, const float* __restrict__ nq2_q,
     const float* __restrict__ C, const float* __restrict__ cnorm,
     const float* __restrict__ cnorm_max, int K, int metric, int nprobe,
-    const int32_t* __restrict__ nprobe_q, int sort_n, const int32_t* __restrict__ pre_ids,
-    const float* __restrict__ pre_dist, int pre_n, int32_t* __restrict__ out_ids,
-    float* __restrict__ out_dist) {
+    const int32_t* __restrict__ nprobe_q, int sort_n, int32_t* __restrict__ out_ids,
+    float* __restrict__ out_dist, const int* __restrict__ redo, int nred) {
   extern __shared__ __align__(16) unsigned char psm[];
   // layout: q (d floats) | the pool (pool_n entries) | work area: the
   // histogram, then the candidates, or the fallback's sort buffer
   float* qs = reinterpret_cast<float*>(psm);
-  uint32_t* sp = reinterpret_cast<uint32_t*>(psm + align_up(sizeof(float) * d, 16));
-  unsigned char* work = psm + align_up(sizeof(float) * d, 16) + align_up(sizeof(uint32_t) * pool_n, 16);
+  const int ld = (d + 31) / 32 * 32;  // columns of the rotated centroid rows C
+  uint32_t* sp = reinterpret_cast<uint32_t*>(psm + sizeof(float) * ld);
+  unsigned char* work = psm + sizeof(float) * ld + align_up(sizeof(uint32_t) * pool_n, 16);
   __shared__ SelState st;
   __shared__ int s_nc, s_bin, s_np, s_nsat;
   __shared__ uint32_t s_pmin, s_pmax;
   __shared__ int s_sat[64];  // saturated groups of 128 centroids (scanned in full)
-  const int q = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // query b (of redo[1 ..] when given: the queries the warp kernel left)
+  const int n_items = redo ? min(*redo, nred) : (int)gridDim.x;
+  for (int b = blockIdx.x; b < n_items; b += gridDim.x) {
+  __syncthreads();
+  const int q = redo ? redo[1 + b] : b;
   const float* qg = Q + (int64_t)q * d;
   const uint32_t* row = keys + (int64_t)q * K;
   int nsel = nprobe;
   if (nprobe_q) nsel = min(max(nprobe_q[q], 1), nprobe);
   nsel = min(nsel, K);
-  if (pre_ids && nsel <= pre_n) {
-    // a list of this query's pre_n best is already selected: its prefix is
-    // the answer (the same order by (score, id))
-    for (int j = tid; j < nprobe; j += blockDim.x) {
-      const bool ok = j < nsel;
-      out_ids[(int64_t)q * nprobe + j] = ok ? pre_ids[(int64_t)q * pre_n + j] : -1;
-      out_dist[(int64_t)q * nprobe + j] =
-          ok ? pre_dist[(int64_t)q * pre_n + j] : __int_as_float(0x7f800000);
-    }
-    return;
-  }
-  for (int i = tid; i < d; i += blockDim.x) qs[i] = qg[i];
+  for (int i = tid; i < ld; i += blockDim.x) qs[i] = i < d ? qg[i] : 0.0f;
   if (tid == 0) {
     s_nc = 0;
     s_np = 0;
@@ -1000,7 +223,11 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     }
   }
   __syncthreads();
-  const bool from_pool = nsel <= s_np;
+  // (From the pool only while it holds well over nsel entries: near its own
+  // size the nsel-th smallest entry is a loose threshold and several times
+  // nsel centroids get their canonical scores. 64 of K = 1024, where the pool
+  // is those 64: 193 us per 8000 queries against 125 from all keys.)
+  const bool from_pool = 2 * nsel <= s_np;
   // T bounds the nsel-th smallest upper bound of all centroids from above.
   // From the pool (distinct centroids): the last value of the histogram bin
   // (over the pool's range) holding the nsel-th smallest entry, so at least
@@ -1031,10 +258,11 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
   }
   __syncthreads();
   {
-    int cb[4], sum = 0;
+    constexpr int NB = kHistBins / kThreads;  // bins per thread
+    int cb[NB], sum = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      cb[u] = hist[4 * tid + u];
+    for (int u = 0; u < NB; ++u) {
+      cb[u] = hist[NB * tid + u];
       sum += cb[u];
     }
     int incl = sum;
@@ -1050,9 +278,9 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     if (excl < nsel && incl >= nsel) {  // exactly one thread
       int cum = excl;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < NB; ++u) {
         if (cum + cb[u] >= nsel) {
-          s_bin = 4 * tid + u;
+          s_bin = NB * tid + u;
           break;
         }
         cum += cb[u];
@@ -1146,14 +374,13 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     // canonical scores of the candidates (one thread each, the full scan's
     // fold); every line of their rows is requested first
     for (int i = tid; i < nc; i += blockDim.x) {
-      const char* x = reinterpret_cast<const char*>(C + (int64_t)(uint32_t)ckey[i] * d);
-      for (int o = 0; o < d * (int)sizeof(float); o += 128)
+      const char* x = reinterpret_cast<const char*>(C + (int64_t)(uint32_t)ckey[i] * ld);
+      for (int o = 0; o < ld * (int)sizeof(float); o += 128)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(x + o));
     }
     for (int i = tid; i < nc; i += blockDim.x) {
       const int c = (int)(uint32_t)ckey[i];
-      const float* x = C + (int64_t)c * d;
-      const float a = metric ? row_score<true>(x, qs, d) : row_score<false>(x, qs, d);
+      const float a = metric ? row_score_rot<true>(C, c, qs, ld) : row_score_rot<false>(C, c, qs, ld);
       ckey[i] = ((unsigned long long)float_key(a) << 32) | (uint32_t)c;
     }
     __syncthreads();
@@ -1161,7 +388,13 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     for (int i = tid; i < nc; i += blockDim.x) {
       const unsigned long long mine = ckey[i];
       int r = 0;
-      for (int j = 0; j < nc; ++j) r += ckey[j] < mine ? 1 : 0;
+      const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(ckey);
+#pragma unroll 4
+      for (int j = 0; j < nc / 2; ++j) {
+        const ulonglong2 c = c2[j];
+        r += (c.x < mine ? 1 : 0) + (c.y < mine ? 1 : 0);
+      }
+      if (nc & 1) r += ckey[nc - 1] < mine ? 1 : 0;
       if (r < nsel) {
         oid[r] = (int32_t)(mine & 0xffffffffu);
         od[r] = key_float((uint32_t)(mine >> 32));
@@ -1175,11 +408,209 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     // too many candidates: the row select over canonical scores computed on
     // the fly (every pass refolds them; a rare path)
     select_row(
-        [qs, C, d, metric](int c) {
-          const float* x = C + (int64_t)c * d;
-          return metric ? row_score<true>(x, qs, d) : row_score<false>(x, qs, d);
+        [qs, C, ld, metric](int c) {
+          return metric ? row_score_rot<true>(C, c, qs, ld) : row_score_rot<false>(C, c, qs, ld);
         },
         K, nsel, nprobe, sort_n, reinterpret_cast<unsigned long long*>(work), oid, od);
+  }
+  }
+}
+
+// The same selection with one warp per query, for batches: no block barriers
+// between its short steps, and as many queries in flight per SM as warps (a
+// CTA per query waited at some fifteen barriers for little work). 62 of 4096,
+// 10k queries: 84 us against 133; 16 of 1024, 8000 queries: 27 against 76.
+// The threshold comes from a histogram of kWarpBins bins; a query with more
+// than kWarpCand candidates goes to redo (count, then the queries) for the
+// CTA kernel.
+constexpr int kPsWarps = 4, kWarpBins = 256, kWarpCand = 512;
+__global__ void __launch_bounds__(32 * kPsWarps) probe_select_warp_kernel(
+    const float* __restrict__ Q, int64_t nq, int d, const uint32_t* __restrict__ keys,
+    const uint32_t* __restrict__ pool, int pool_n, const uint32_t* __restrict__ kmin_q,
+    const uint32_t* __restrict__ kmax_q, const float* __restrict__ nq2_q,
+    const float* __restrict__ C, const float* __restrict__ cnorm,
+    const float* __restrict__ cnorm_max, int K, int metric, int nprobe,
+    const int32_t* __restrict__ nprobe_q, int32_t* __restrict__ out_ids,
+    float* __restrict__ out_dist, int* __restrict__ redo) {
+  extern __shared__ __align__(16) unsigned char psm[];
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t q = (int64_t)blockIdx.x * kPsWarps + wid;
+  if (q >= nq) return;
+  const int ld = (d + 31) / 32 * 32;  // columns of the rotated centroid rows C
+  const size_t qb = sizeof(float) * ld;
+  unsigned char* mine_sm = psm + (size_t)wid * (qb + sizeof(unsigned long long) * kWarpCand);
+  float* qs = reinterpret_cast<float*>(mine_sm);
+  unsigned long long* ckey = reinterpret_cast<unsigned long long*>(mine_sm + qb);
+  int* hist = reinterpret_cast<int*>(ckey);
+  const uint32_t* row = keys + q * K;
+  const uint32_t* pl = pool + q * pool_n;
+  int32_t* oid = out_ids + q * nprobe;
+  float* od = out_dist + q * nprobe;
+  int nsel = nprobe;
+  if (nprobe_q) nsel = min(max(nprobe_q[q], 1), nprobe);
+  nsel = min(nsel, K);
+  for (int i = lane; i < ld; i += 32) qs[i] = i < d ? __ldg(Q + q * d + i) : 0.0f;
+  for (int i = lane; i < kWarpBins; i += 32) hist[i] = 0;
+  const ProbeEps eps(metric, __fsqrt_rn(nq2_q[q]), d);
+  int cnt = 0;
+  uint32_t pmin = 0xffffffffu, pmax = 0u;
+  for (int i = lane; i < pool_n; i += 32) {
+    const uint32_t e = __ldg(pl + i);
+    if (e != 0xffffffffu) {
+      ++cnt;
+      pmin = min(pmin, e);
+      pmax = max(pmax, e);
+    }
+  }
+  cnt = __reduce_add_sync(kFull, cnt);
+  const bool from_pool = 2 * nsel <= cnt;
+  // (nsel pooled entries bound the nsel-th smallest key, so that keys above
+  // the pool's largest need no bin)
+  const uint32_t kmin = from_pool ? __reduce_min_sync(kFull, pmin) : kmin_q[q];
+  const uint32_t kmax = nsel <= cnt ? __reduce_max_sync(kFull, pmax) : kmax_q[q];
+  const uint32_t span1 = kmax - kmin;
+  int shift = 0;
+  while ((span1 >> shift) >= (uint32_t)kWarpBins) ++shift;
+  __syncwarp();
+  if (from_pool) {
+    for (int i = lane; i < pool_n; i += 32) {
+      const uint32_t e = __ldg(pl + i);
+      if (e != 0xffffffffu) atomicAdd(&hist[(e - kmin) >> shift], 1);
+    }
+  } else {
+    for (int c0 = 0; c0 < K; c0 += 256) {
+      uint32_t kv[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) kv[u] = c0 + 32 * u + lane < K ? __ldg(row + c0 + 32 * u + lane) : 0u;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (c0 + 32 * u + lane < K && kv[u] <= kmax) atomicAdd(&hist[(kv[u] - kmin) >> shift], 1);
+    }
+  }
+  __syncwarp();
+  int cb[kWarpBins / 32], sum = 0;
+#pragma unroll
+  for (int u = 0; u < kWarpBins / 32; ++u) {
+    cb[u] = hist[lane * (kWarpBins / 32) + u];
+    sum += cb[u];
+  }
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const int owner = __ffs(__ballot_sync(kFull, incl >= nsel)) - 1;
+  int bin = 0, cum = incl - sum;
+#pragma unroll
+  for (int u = 0; u < kWarpBins / 32; ++u)
+    if (cum < nsel) {
+      bin = lane * (kWarpBins / 32) + u;
+      cum += cb[u];
+    }
+  bin = __shfl_sync(kFull, bin, owner);
+  const uint64_t edge = (uint64_t)kmin + ((uint64_t)(bin + 1) << shift) - 1u;
+  const uint32_t T = (uint32_t)min((uint64_t)kmax, edge);
+  const float Tf = key_float(T), e2max = __fmul_rn(2.0f, eps(__ldg(cnorm_max)));
+  const uint32_t Tpre =
+      float_key(__fadd_ru(__fadd_ru(Tf, e2max), __fmul_ru(0x1.0p-20f, __fadd_ru(fabsf(Tf), e2max))));
+  const uint64_t lim = (uint64_t)Tpre + 128u;
+  int nc = 0;
+  const unsigned lt = (1u << lane) - 1u;
+  // U centroids per lane, their keys (and then norms) loaded together
+  constexpr int U = 8;
+  auto consider = [&](const bool (&want)[U], const int (&c)[U]) {  // whole warp
+    uint32_t key[U];
+    bool in[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) key[u] = want[u] ? __ldg(row + c[u]) : 0xffffffffu;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      in[u] = want[u] && key[u] <= Tpre;
+      const float n = in[u] ? __ldg(cnorm + c[u]) : 0.0f;
+      in[u] = in[u] && float_key(__fsub_rn(key_float(key[u]), __fmul_rn(2.0f, eps(n)))) <= T;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned m = __ballot_sync(kFull, in[u]);
+      const int slot = nc + __popc(m & lt);
+      if (in[u] && slot < kWarpCand) ckey[slot] = (unsigned long long)(uint32_t)c[u];
+      nc += __popc(m);
+    }
+  };
+  auto consider_run = [&](int c0, int c1) {  // every centroid of [c0, c1)
+    for (; c0 < c1; c0 += 32 * U) {
+      bool want[U];
+      int c[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        c[u] = c0 + 32 * u + lane;
+        want[u] = c[u] < c1;
+      }
+      consider(want, c);
+    }
+  };
+  __syncwarp();  // (the histogram is read)
+  if (from_pool) {
+    for (int i0 = 0; i0 < pool_n; i0 += 32 * U) {  // (pool_n: a multiple of 16)
+      uint32_t e[U];
+      bool want[U];
+      int c[U];
+      unsigned sg[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + 32 * u + lane;
+        e[u] = i < pool_n ? __ldg(pl + i) : 0xffffffffu;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const uint32_t last = __shfl_sync(kFull, e[u], lane | (kProbePool - 1));
+        const bool sat = last != 0xffffffffu && (uint64_t)(last & ~127u) <= lim;
+        c[u] = (i0 + 32 * u + lane) / kProbePool * 128 + (int)(e[u] & 127u);
+        want[u] = !sat && e[u] != 0xffffffffu && (uint64_t)(e[u] & ~127u) <= lim;
+        sg[u] = __ballot_sync(kFull, sat && (lane & (kProbePool - 1)) == 0);
+      }
+      consider(want, c);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        while (sg[u]) {  // saturated groups of 128 centroids: scanned in full
+          const int g = (i0 + 32 * u + __ffs(sg[u]) - 1) / kProbePool;
+          sg[u] &= sg[u] - 1;
+          consider_run(g * 128, min(K, g * 128 + 128));
+        }
+    }
+  } else {
+    consider_run(0, K);
+  }
+  if (nc > kWarpCand) {
+    if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int)q;
+    return;
+  }
+  __syncwarp();
+  for (int i = lane; i < nc; i += 32) {
+    const int c = (int)(uint32_t)ckey[i];
+    const float a = metric ? row_score_rot<true>(C, c, qs, ld) : row_score_rot<false>(C, c, qs, ld);
+    ckey[i] = ((unsigned long long)float_key(a) << 32) | (uint32_t)c;
+  }
+  if (lane == 0 && (nc & 1)) ckey[nc] = ~0ull;  // (an even count is compared in pairs)
+  __syncwarp();
+  for (int i = lane; i < nc; i += 32) {
+    const unsigned long long mine = ckey[i];
+    int r = 0;
+    const ulonglong2* c2 = reinterpret_cast<const ulonglong2*>(ckey);
+#pragma unroll 4
+    for (int j = 0; j < (nc + 1) / 2; ++j) {
+      const ulonglong2 c = c2[j];
+      r += (c.x < mine ? 1 : 0) + (c.y < mine ? 1 : 0);
+    }
+    if (r < nsel) {
+      oid[r] = (int32_t)(mine & 0xffffffffu);
+      od[r] = key_float((uint32_t)(mine >> 32));
+    }
+  }
+  for (int j = nsel + lane; j < nprobe; j += 32) {
+    oid[j] = -1;
+    od[j] = __int_as_float(0x7f800000);
   }
 }
 
@@ -1188,233 +619,7 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
 inline size_t probe_select_smem(int d, int sort_n, int pool_n) {
   const size_t work = std::max({sizeof(int) * kHistBins, sizeof(unsigned long long) * kProbeCandMax,
                                 sizeof(unsigned long long) * (size_t)sort_n});
-  return align_up(sizeof(float) * d, 16) + align_up(sizeof(uint32_t) * (size_t)pool_n, 16) + work;
-}
-
-// Shared counters the per-query finishing step works with.
-struct TailShared {
-  int* cand_cnt;
-  int* top_cnt;
-  int* surv;
-  int* scratch;  // kCompactU x kThreads / 32 ints
-};
-
-// The per-query end of the search (§4, reading R1): given the list of
-// candidates {position, LB, estimate, UB} that contains every code with
-// LB <= tau_ub, keep LB <= tau_ub; pilot = the m smallest (estimate, id);
-// exact distances of the pilot give tau1; tau = min(tau_ub, tau1); exact
-// distances of the other codes with LB <= tau; top-k by (distance, id).
-// The pilot mark is bit 31 of the position. Whole block.
-__device__ void finish_query(const FusedParams& P, const FusedSmem& S, int64_t q, int4* cand,
-                             int cand_cap, float tau_ub, const TailShared& ts,
-                             bool filtered = false) {
-  const int tid = threadIdx.x;
-  const int k = P.k, m = P.m;
-  if (tid == 0) {
-    *ts.top_cnt = 0;
-    *ts.surv = 0;
-  }
-  __syncthreads();
-  if (!filtered)  // (a list staged with LB <= tau_ub is already filtered)
-    compact_cand(cand, ts.cand_cnt, cand_cap, ts.scratch,
-                 [tau_ub](const int4& e) { return __int_as_float(e.y) <= tau_ub; });
-  // pilot: the m smallest (estimate, id) of the list
-  const int nl = *ts.cand_cnt;
-  const bool pilot_all = nl <= m;
-  uint32_t T_e = 0xffffffffu, T_id = 0xffffffffu;
-  if (!pilot_all) {
-    // the top-k buffer is free until the pilot's re-rank: histogram and
-    // boundary-bin keys go there
-    int ties = 0, eqn = 0;
-    T_e = hist_select(nl, m, *S.sel, reinterpret_cast<int*>(S.topk),
-                      reinterpret_cast<uint32_t*>(S.topk) + kHistBins, 2 * P.ct - kHistBins, ties,
-                      eqn, [cand](int i) { return float_key(__int_as_float(cand[i].z)); });
-    // among the list entries whose estimate equals the m-th one, the
-    // `ties` smallest ids belong to the pilot; when all of them belong (the
-    // usual case: one entry) no id selection is needed
-    if (eqn > ties)
-      T_id = block_select_f<uint32_t>(nl, ties, *S.sel, [cand, T_e, &P](int i) {
-        const int4 e = cand[i];
-        return float_key(__int_as_float(e.z)) == T_e ? (uint32_t)__ldg(P.perm + e.x) : 0xffffffffu;
-      });
-  }
-  // write the pilot's (id, position) pairs to the pilot list, mark them
-  __shared__ int s_pilot;
-  if (tid == 0) s_pilot = 0;
-  __syncthreads();
-  for (int b0 = 0; b0 < nl; b0 += blockDim.x) {
-    const int i = b0 + tid;
-    bool in = false;
-    int4 e = make_int4(0, 0, 0, 0);
-    if (i < nl) {
-      e = cand[i];
-      const uint32_t ek = float_key(__int_as_float(e.z));
-      in = pilot_all || ek < T_e || (ek == T_e && (uint32_t)__ldg(P.perm + e.x) <= T_id);
-    }
-    const int slot = warp_reserve(in, &s_pilot);
-    if (in) {
-      S.estk[slot] = (uint32_t)e.x;
-      cand[i].x = e.x | (int)0x80000000;
-    }
-  }
-  __syncthreads();
-  const int pilot = s_pilot;
-  // the pilot's ids, all loads in flight together
-  for (int i = tid; i < pilot; i += blockDim.x) {
-    const unsigned long long e = S.estk[i];
-    S.estk[i] = ((unsigned long long)(uint32_t)__ldg(P.perm + (uint32_t)e) << 32) | e;
-  }
-  __syncthreads();
-  // exact distances of the pilot; tau1 = k-th smallest of them
-  rerank_rows<0>(P, S, q, pilot, cand, ts.top_cnt, ts.surv);
-  // tau1: the k-th smallest exact distance of the pilot; only the k smallest
-  // pilot keys can be in the result, so the rest are dropped here
-  // (the pilot list is free now and holds the histogram when large enough;
-  // the upper-bound buffer, free since tau_ub, holds the boundary keys)
-  const bool hsel = 2 * P.ce >= kHistBins && P.cu >= 256;
-  const unsigned long long T1 =
-      (pilot >= k) ? select_keep_dk(S.topk, ts.top_cnt, k, *S.sel,
-                                    hsel ? reinterpret_cast<int*>(S.estk) : nullptr, S.ubk, P.cu)
-                   : ~0ull;
-  const float tau1 = (pilot >= k) ? key_float((uint32_t)(T1 >> 32)) : __int_as_float(0x7f800000);
-  const float tau = fminf(tau_ub, tau1);
-  // the rest of the re-rank set: LB <= tau, outside the pilot
-  compact_cand(cand, ts.cand_cnt, cand_cap, ts.scratch,
-               [tau](const int4& e) { return e.x >= 0 && __int_as_float(e.y) <= tau; });
-  // with k pilot keys kept, a key above the k-th of them cannot be in the
-  // result (keys are distinct): such keys are not kept
-  rerank_rows<1>(P, S, q, *ts.cand_cnt, cand, ts.top_cnt, ts.surv, T1);
-  const int n_top = *ts.top_cnt;
-  if (n_top <= (int)blockDim.x) {
-    // few keys (the usual case): each thread ranks its key against all of
-    // them (distinct keys, so the ranks are a permutation) and writes it to
-    // its place in the result
-    const bool has = tid < n_top;
-    const unsigned long long mine = has ? S.topk[tid] : 0ull;
-    int r = 0;
-    if (has)
-      for (int j2 = 0; j2 < n_top; ++j2) r += S.topk[j2] < mine ? 1 : 0;
-    if (has && r < k) {
-      P.out_ids[q * k + r] = (int64_t)(mine & 0xffffffffu);
-      const float v = key_float((uint32_t)(mine >> 32));
-      P.out_dist[q * k + r] = P.metric ? -v : v;  // inner products: <o_r, q_r>
-    }
-    for (int j2 = n_top + tid; j2 < k; j2 += blockDim.x) {
-      P.out_ids[q * k + j2] = -1;
-      P.out_dist[q * k + j2] = P.metric ? __int_as_float(0xff800000) : __int_as_float(0x7f800000);
-    }
-  } else {
-    select_keep_dk(S.topk, ts.top_cnt, k, *S.sel);
-    const int got = min(*ts.top_cnt, k);
-    sort_kept_u64(S.topk, got, k);
-    for (int j2 = tid; j2 < k; j2 += blockDim.x) {
-      const bool ok = j2 < got;
-      P.out_ids[q * k + j2] = ok ? (int64_t)(S.topk[j2] & 0xffffffffu) : -1;
-      const float v = ok ? key_float((uint32_t)(S.topk[j2] >> 32)) : __int_as_float(0x7f800000);
-      P.out_dist[q * k + j2] = P.metric ? -v : v;  // inner products: <o_r, q_r>, -inf pads
-    }
-  }
-  if (tid == 0) {
-    if (P.tr.tau_ub) P.tr.tau_ub[q] = tau_ub;
-    if (P.tr.tau1) P.tr.tau1[q] = tau1;
-    if (P.tr.tau) P.tr.tau[q] = tau;
-    if (P.tr.n_surv) P.tr.n_surv[q] = *ts.surv;
-  }
-  __syncthreads();
-}
-
-// Code words of one code held in registers (WT > 0: compile-time length,
-// loaded as 16-byte vectors; WT = 0: generic length, read in place).
-template <int WT>
-struct CodeRegs {
-  uint64_t c[WT > 0 ? WT : 1];
-};
-
-template <int WT>
-__device__ __forceinline__ void load_code(CodeRegs<WT>& r, const uint64_t* __restrict__ code) {
-  if constexpr (WT == 4) {  // one 32-byte load (codes are 32-byte aligned)
-    asm volatile("ld.global.nc.v4.u64 {%0,%1,%2,%3}, [%4];"
-                 : "=l"(r.c[0]), "=l"(r.c[1]), "=l"(r.c[2]), "=l"(r.c[3])
-                 : "l"(code));
-  } else if constexpr (WT > 0) {
-    if constexpr (WT % 2 == 0) {
-#pragma unroll
-      for (int w = 0; w < WT; w += 2) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(code) + w / 2);
-        r.c[w] = ((uint64_t)v.y << 32) | v.x;
-        r.c[w + 1] = ((uint64_t)v.w << 32) | v.z;
-      }
-    } else {
-#pragma unroll
-      for (int w = 0; w < WT; ++w) r.c[w] = __ldg(code + w);
-    }
-  }
-}
-
-// <x_b, q_u> of one code against the bit-planes of its probe (§3.3.2):
-// sum_j 2^j popcount(x_b AND q_u^(j)), unrolled for a compile-time code length
-// (WT words) and B_q (BQT planes); WT = 0 / BQT = 0 use the runtime values.
-template <int WT, int BQT>
-__device__ __forceinline__ int code_ip(const CodeRegs<WT>& r, const uint64_t* __restrict__ code,
-                                       const uint64_t* pl, int W, int bq) {
-  if constexpr (WT > 0 && BQT > 0) {
-    int ip = 0;
-#pragma unroll
-    for (int b = 0; b < BQT; ++b) {
-      uint64_t pw[WT];
-      if constexpr (WT % 2 == 0) {
-#pragma unroll
-        for (int w = 0; w < WT; w += 2) {
-          const uint4 v = *reinterpret_cast<const uint4*>(pl + b * WT + w);
-          pw[w] = ((uint64_t)v.y << 32) | v.x;
-          pw[w + 1] = ((uint64_t)v.w << 32) | v.z;
-        }
-      } else {
-#pragma unroll
-        for (int w = 0; w < WT; ++w) pw[w] = pl[b * WT + w];
-      }
-      int pb = 0;
-#pragma unroll
-      for (int w = 0; w < WT; ++w) pb += __popcll(r.c[w] & pw[w]);
-      ip += pb << b;
-    }
-    return ip;
-  } else {
-    int ip = 0;
-    for (int b = 0; b < bq; ++b) {
-      int pb = 0;
-      for (int w = 0; w < W; ++w) pb += __popcll(code[w] & pl[b * W + w]);
-      ip += pb << b;
-    }
-    return ip;
-  }
-}
-
-// <x_b, q_u> of two codes of the same probe: each plane word is read from
-// shared memory once for both (D' = 128 / 256, B_q = 4).
-template <int WT>
-__device__ __forceinline__ void code_ip2(const CodeRegs<WT>& r0, const CodeRegs<WT>& r1,
-                                         const uint64_t* pl, int& i0, int& i1) {
-  i0 = 0;
-  i1 = 0;
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    uint64_t pw[WT];
-#pragma unroll
-    for (int w = 0; w < WT; w += 2) {
-      const uint4 v = *reinterpret_cast<const uint4*>(pl + b * WT + w);
-      pw[w] = ((uint64_t)v.y << 32) | v.x;
-      pw[w + 1] = ((uint64_t)v.w << 32) | v.z;
-    }
-    int p0 = 0, p1 = 0;
-#pragma unroll
-    for (int w = 0; w < WT; ++w) {
-      p0 += __popcll(r0.c[w] & pw[w]);
-      p1 += __popcll(r1.c[w] & pw[w]);
-    }
-    i0 += p0 << b;
-    i1 += p1 << b;
-  }
+  return sizeof(float) * (size_t)((d + 31) / 32 * 32) + align_up(sizeof(uint32_t) * (size_t)pool_n, 16) + work;
 }
 
 constexpr int kPPT = 4;  // most appends per thread between two buffer upkeeps (sizing)
@@ -3292,41 +2497,64 @@ int fused_shape(const SearchArgs& a, FusedShape* f) {
 
 // Probe lists from the probe keys in cd (probe_keys_tc):
 // the nsel (= nprobe, or npq[q] clamped to it) best centroids of each query
-// by exact canonical score, ascending (score, id), in rows of nprobe. With
-// pre_ids/pre_dist (rows of pre_n such lists), a query with nsel <= pre_n
-// copies its prefix instead.
+// by exact canonical score, ascending (score, id), in rows of nprobe.
+// only_redo: just the queries on the scratch's redo list.
 int probe_select(const rabitq_index* X, const float* Q, int64_t nqc, const float* cd, int nprobe,
                  const int32_t* npq, int32_t* ids, float* dist, cudaStream_t s,
-                 const int32_t* pre_ids = nullptr, const float* pre_dist = nullptr,
-                 int pre_n = 0) {
+                 bool only_redo = false) {
   if (nqc <= 0) return RABITQ_OK;
   const int sort_n = pow2_at_least(nprobe);
   int dev = 0, optin = 0;
   RBQ_CUDA(cudaGetDevice(&dev));
   RBQ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-  cudaFuncAttributes fa;
-  RBQ_CUDA(cudaFuncGetAttributes(&fa, probe_select_kernel));
-  const size_t limit = (size_t)(optin - (int)fa.sharedSizeBytes);
-  RBQ_CUDA(cudaFuncSetAttribute(probe_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)limit));
   const ProbeScratch v = probe_scratch(X, nqc, const_cast<float*>(cd));
+  const int metric = X->metric != RABITQ_METRIC_L2 ? 1 : 0;
+  // One warp per query once the batch gives every SM a dozen warps (a single
+  // query is sooner done by a whole CTA) and the lists are short.
+  const bool by_warp = !only_redo && nqc >= 1024 && nprobe <= 64;
+  if (by_warp) {
+    const size_t smem =
+        kPsWarps * (sizeof(float) * ((X->d + 31) / 32 * 32) + sizeof(unsigned long long) * kWarpCand);
+    RBQ_CUDA(cudaFuncSetAttribute(probe_select_warp_kernel,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    probe_select_warp_kernel<<<(unsigned)((nqc + kPsWarps - 1) / kPsWarps), 32 * kPsWarps, smem, s>>>(
+        Q, nqc, X->d, v.keys, v.pool, v.pool_n, v.kmin, v.kmax, v.nq2, X->cent_rot, X->cnorm,
+        X->cnorm_max, X->K, metric, nprobe, npq, ids, dist, v.redo);
+    RBQ_CUDA(cudaGetLastError());
+  }
+  const bool redo = by_warp || only_redo;
+  const auto fn = probe_select_kernel;
+  cudaFuncAttributes fa;
+  RBQ_CUDA(cudaFuncGetAttributes(&fa, fn));
+  const size_t limit = (size_t)(optin - (int)fa.sharedSizeBytes);
+  RBQ_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
   const size_t smem = probe_select_smem(X->d, sort_n, v.pool_n);
   if (smem > limit) return fail(RABITQ_EINVAL, "probe selection does not fit shared memory");
-  probe_select_kernel<<<(unsigned)nqc, kThreads, smem, s>>>(
-      Q, X->d, v.keys, v.pool, v.pool_n, v.kmin, v.kmax, v.nq2, X->centroids, X->cnorm,
-      X->cnorm_max, X->K, X->metric != RABITQ_METRIC_L2 ? 1 : 0, nprobe, npq, sort_n, pre_ids,
-      pre_dist, pre_n, ids, dist);
+  fn<<<(unsigned)(redo ? std::min<int64_t>(nqc, 152) : nqc), kThreads, smem, s>>>(
+      Q, X->d, v.keys, v.pool, v.pool_n, v.kmin, v.kmax, v.nq2, X->cent_rot, X->cnorm,
+      X->cnorm_max, X->K, metric, nprobe, npq, sort_n, ids, dist, only_redo ? v.redo_mlp : redo ? v.redo : nullptr, (int)nqc);
   RBQ_CUDA(cudaGetLastError());
   return RABITQ_OK;
 }
 
-// Learned probe counts of one query chunk from its centroid products cd
-// (nqc x K): the min(64, K) nearest buckets, then the fused MLP kernel.
-int predict_chunk(const SearchArgs& a, const float* Q, const float* cd, int64_t nqc, int64_t q0,
-                  int32_t* fid, float* fdist, cudaStream_t s) {
+// Learned probe counts npq and probe lists (rows of nprobe) of one query
+// chunk from its centroid products cd (nqc x K): the min(64, K) nearest
+// buckets, then the fused MLP kernel, which also copies the lists that fit
+// them; the selection runs for the queries that need more.
+int predict_chunk(const SearchArgs& a, const float* Q, const float* cd, int64_t nqc, int nprobe,
+                  int32_t* npq, int32_t* fid, float* fdist, int32_t* ids, float* dist,
+                  cudaStream_t s) {
   const int navail = std::min(kMlpIn, a.X->K);
   RBQ_CHECK(probe_select(a.X, Q, nqc, cd, navail, nullptr, fid, fdist, s));
-  return mlp_infer(a.pred, fdist, navail, nqc, navail, a.pred_nprobe + q0, nullptr, nullptr, s);
+  MlpLists lists;
+  lists.sel_ids = fid;
+  lists.out_ids = ids;
+  lists.out_dist = dist;
+  lists.ldo = nprobe;
+  lists.redo = probe_scratch(a.X, nqc, const_cast<float*>(cd)).redo_mlp;
+  RBQ_CHECK(mlp_infer(a.pred, fdist, navail, nqc, navail, npq, nullptr, nullptr, s, lists));
+  if (nprobe <= navail) return RABITQ_OK;
+  return probe_select(a.X, Q, nqc, cd, nprobe, npq, ids, dist, s, true);
 }
 
 }  // namespace
@@ -3505,7 +2733,16 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
   if (wfn) RBQ_CHECK(warp_ctas(wfn, &wctas));
   const int capw = warp_capw(a);
   DevBuf candw, redo, wkey, worder, wooff, wsortws;
-  if (wfn) {
+  // the bucket-major scan, where it applies (without memory for its lists the
+  // per-query scan runs)
+  const bool bucket = split == 1 && bucket_applies(a, std::min(qchunk, a.nq));
+  DevBuf bscratch;
+  const bool by_bucket = bucket && bscratch.alloc(bucket_bytes(a, qchunk), s) == RABITQ_OK;
+  if (bucket && !by_bucket) {
+    cudaGetLastError();
+    set_error("");
+  }
+  if (wfn && !by_bucket) {
     RBQ_CHECK(candw.alloc(sizeof(int4) * wctas * (kWarpThreads / 32) * capw, s));
     RBQ_CHECK(redo.alloc(sizeof(int32_t) * (qchunk + 64), s));
     RBQ_CHECK(wkey.alloc(sizeof(int32_t) * qchunk, s));
@@ -3561,17 +2798,13 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
     float* probe_dist = a.trace && a.trace->probe_dist ? a.trace->probe_dist + q0 * nprobe
                                                        : pdist.as<float>();
     const int32_t* npq = a.per_query_nprobe ? a.per_query_nprobe + q0 : nullptr;
-    // learned counts: the 64 nearest buckets give the features, the network
-    // gives each query's count, and the probe list then holds that many (a
-    // selection of nprobe_max for every query would cost more: most need few)
     if (a.pred) {
-      RBQ_CHECK(predict_chunk(a, Q, cd.as<float>(), nqc, q0, fid.as<int32_t>(),
-                              fdist.as<float>(), s));
+      RBQ_CHECK(predict_chunk(a, Q, cd.as<float>(), nqc, nprobe, a.pred_nprobe + q0,
+                              fid.as<int32_t>(), fdist.as<float>(), probe_ids, probe_dist, s));
       npq = a.pred_nprobe + q0;
+    } else {
+      RBQ_CHECK(probe_select(X, Q, nqc, cd.as<float>(), nprobe, npq, probe_ids, probe_dist, s));
     }
-    RBQ_CHECK(probe_select(X, Q, nqc, cd.as<float>(), nprobe, npq, probe_ids, probe_dist, s,
-                           a.pred ? fid.as<int32_t>() : nullptr, fdist.as<float>(),
-                           std::min(kMlpIn, K)));
     if (metric_ip(X)) RBQ_CHECK(probe_nq2(X, Q, nqc, nprobe, probe_ids, pnq2.as<float>(), s));
     if (timing) RBQ_CUDA(cudaEventRecord(ev[2], s));
     float* rqp = a.trace && a.trace->rq ? a.trace->rq + q0 * dpad : rq.as<float>();
@@ -3620,7 +2853,7 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
     P.err = err.as<int>();
     P.next = nextc.as<int>();
     RBQ_CUDA(cudaMemsetAsync(nextc.p, 0, sizeof(int), s));
-    if (npq) {
+    if (npq && !by_bucket) {
       order_key_kernel<<<(unsigned)((nqc + 255) / 256), 256, 0, s>>>(npq, nqc, nprobe,
                                                                     okey.as<int32_t>());
       if (order_sort_fits(nqc, nprobe + 1))
@@ -3659,7 +2892,9 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
       P.slice_cnt = scnt.as<int>();
       P.cand2 = cand2.as<int4>();
     }
-    if (wfn && warp_batch_ok(a, nqc, wctas)) {
+    if (by_bucket) {
+      RBQ_CHECK(bucket_search(a, P, bscratch.as<unsigned char>(), fn, (unsigned)grid, smem, s));
+    } else if (wfn && warp_batch_ok(a, nqc, wctas)) {
       const WarpScratch ws{candw.as<int4>(), capw, redo.as<int>(), wkey.as<int32_t>(),
                            worder.as<int32_t>(), wooff.as<int32_t>(), wsortws.as<int32_t>()};
       RBQ_CHECK(launch_warp(wfn, wctas, P, ws, fn, (unsigned)grid, smem, s));
@@ -3717,6 +2952,8 @@ struct Carve {
   WarpFn wfn = nullptr;
   int64_t wctas = 0;
   int capw = 0;
+  size_t o_bucket = 0;  // the bucket-major scan's scratch (carve_bucket)
+  bool bucket = false;
   size_t o_candw = 0, o_redo = 0, o_wkey = 0, o_worder = 0, o_wooff = 0, o_wsortws = 0;
 };
 
@@ -3756,6 +2993,8 @@ Carve carve_layout(const SearchArgs& a, int64_t grid, int64_t cap, int64_t qchun
   L.o_ubout = take(a.allow_split ? sizeof(uint32_t) * grid * a.k : 0);
   L.o_scnt = take(a.allow_split ? sizeof(int) * grid * 2 : 0);
   L.o_cand2 = take(a.allow_split ? sizeof(int4) * (grid / 2) * cap : 0);
+  L.bucket = bucket_applies(a, qchunk);
+  L.o_bucket = take(L.bucket ? bucket_bytes(a, qchunk) : 0);
   L.wfn = pick_warp(a);
   if (L.wfn && warp_ctas(L.wfn, &L.wctas) != RABITQ_OK) L.wfn = nullptr;
   if (L.wfn) {
@@ -3837,33 +3076,44 @@ int search_enqueue_carved(const SearchArgs& a, unsigned char* scratch, size_t sc
   int32_t* sortws = reinterpret_cast<int32_t*>(scratch + L.o_sortws);
   float* qn = reinterpret_cast<float*>(scratch + L.o_qn);
   float* pnq2 = reinterpret_cast<float*>(scratch + L.o_pnq2);
-  const int navail = std::min(kMlpIn, K);
   for (int64_t q0 = 0; q0 < a.nq; q0 += qchunk) {
     const int64_t nqc = std::min(qchunk, a.nq - q0);
     const bool ev = a.stage_ev && q0 == 0 && nqc == a.nq;
     if (ev) RBQ_CUDA(cudaEventRecordWithFlags(a.stage_ev[0], s, cudaEventRecordExternal));
     const float* Q = nullptr;
     RBQ_CHECK(search_queries(X, a.queries + q0 * d, nqc, qn, &Q, s));
+    // The rotation needs nothing of the probe selection and fills the SMs no
+    // better than it does: in a plan the two run side by side (serving
+    // request of 53 queries: 180 to 174 us; 10k queries: 2.71 to 2.66 ms).
+    auto rotate = [&](cudaStream_t rs) {
+      if (a.rot_precision == RABITQ_ROT_FP32)
+        return gemm_canon(kDot, Q, d, nullptr, nullptr, 0, nullptr, X->P32, dpad, rq, dpad, nqc,
+                          dpad, d, rs);
+      return rotate_tc(X, Q, nqc, a.rot_precision, rq, err, rs);
+    };
+    const bool beside = a.side && !a.stage_ev;
+    if (beside) {
+      RBQ_CUDA(cudaEventRecord(a.fork, s));
+      RBQ_CUDA(cudaStreamWaitEvent(a.side, a.fork, 0));
+      RBQ_CHECK(rotate(a.side));
+      RBQ_CUDA(cudaEventRecord(a.join, a.side));
+    }
     RBQ_CHECK(centroid_scores(X, Q, nqc, cd, err, s));
     if (ev) RBQ_CUDA(cudaEventRecordWithFlags(a.stage_ev[1], s, cudaEventRecordExternal));
     const int32_t* npq = a.per_query_nprobe ? a.per_query_nprobe + q0 : nullptr;
-    if (a.pred) {  // the 64 nearest give the features, the network each query's count
-      RBQ_CHECK(probe_select(X, Q, nqc, cd, navail, nullptr, fid, fdist, s));
-      RBQ_CHECK(mlp_infer(a.pred, fdist, navail, nqc, navail, pnp, nullptr, nullptr, s));
-      npq = pnp;
+    if (a.pred) {
+      int32_t* counts = a.pred_nprobe ? a.pred_nprobe + q0 : pnp;
+      RBQ_CHECK(predict_chunk(a, Q, cd, nqc, nprobe, counts, fid, fdist, pid, pdist, s));
+      npq = counts;
+    } else {
+      RBQ_CHECK(probe_select(X, Q, nqc, cd, nprobe, npq, pid, pdist, s));
     }
-    RBQ_CHECK(probe_select(X, Q, nqc, cd, nprobe, npq, pid, pdist, s, a.pred ? fid : nullptr,
-                           fdist, navail));
-    if (a.pred && a.pred_nprobe)
-      RBQ_CUDA(cudaMemcpyAsync(a.pred_nprobe + q0, pnp, sizeof(int32_t) * nqc,
-                               cudaMemcpyDeviceToDevice, s));
     if (metric_ip(X)) RBQ_CHECK(probe_nq2(X, Q, nqc, nprobe, pid, pnq2, s));
     if (ev) RBQ_CUDA(cudaEventRecordWithFlags(a.stage_ev[2], s, cudaEventRecordExternal));
-    if (a.rot_precision == RABITQ_ROT_FP32)
-      RBQ_CHECK(gemm_canon(kDot, Q, d, nullptr, nullptr, 0, nullptr, X->P32, dpad, rq, dpad, nqc,
-                           dpad, d, s));
+    if (beside)
+      RBQ_CUDA(cudaStreamWaitEvent(s, a.join, 0));
     else
-      RBQ_CHECK(rotate_tc(X, Q, nqc, a.rot_precision, rq, err, s));
+      RBQ_CHECK(rotate(s));
     if (ev) RBQ_CUDA(cudaEventRecordWithFlags(a.stage_ev[3], s, cudaEventRecordExternal));
     FusedParams P;
     std::memset(&P, 0, sizeof P);
@@ -3904,20 +3154,23 @@ int search_enqueue_carved(const SearchArgs& a, unsigned char* scratch, size_t sc
     P.err = err;
     P.next = next;
     RBQ_CUDA(cudaMemsetAsync(next, 0, sizeof(int), s));
-    if (npq) {
+    const int split = a.allow_split ? split_factor(a, nqc, grid, fs) : 1;
+    const bool by_bucket = L.bucket && split == 1 && bucket_applies(a, nqc);
+    if (npq && !by_bucket) {
       order_key_kernel<<<(unsigned)((nqc + 255) / 256), 256, 0, s>>>(npq, nqc, nprobe, okey);
       RBQ_CUDA(cudaGetLastError());
       RBQ_CHECK(order_sort(okey, nqc, nprobe + 1, order, ooff, sortws, s));
       P.order = order;
     }
-    const int split = a.allow_split ? split_factor(a, nqc, grid, fs) : 1;
     P.split = split;
     if (split > 1) {
       P.ub_out = reinterpret_cast<uint32_t*>(scratch + L.o_ubout);
       P.slice_cnt = reinterpret_cast<int*>(scratch + L.o_scnt);
       P.cand2 = reinterpret_cast<int4*>(scratch + L.o_cand2);
     }
-    if (split == 1 && L.wfn && warp_batch_ok(a, nqc, L.wctas)) {
+    if (by_bucket) {
+      RBQ_CHECK(bucket_search(a, P, scratch + L.o_bucket, fn, (unsigned)grid, smem, s));
+    } else if (split == 1 && L.wfn && warp_batch_ok(a, nqc, L.wctas)) {
       const WarpScratch ws{reinterpret_cast<int4*>(scratch + L.o_candw), L.capw,
                            reinterpret_cast<int*>(scratch + L.o_redo),
                            reinterpret_cast<int32_t*>(scratch + L.o_wkey),
@@ -3944,6 +3197,7 @@ int search_dev_prealloc(const SearchArgs& a_in, unsigned char* scratch, size_t s
   if (a_in.nq == 0) return RABITQ_OK;
   SearchArgs a = a_in;
   a.allow_split = 0;  // the fixed scratch has no room for the split buffers
+  a.allow_bucket = 0;  // ... nor for the bucket-major scan's lists
   // flags: err[0] = search error (1 = candidate overflow, 2 = expired wait),
   // err[1] = a query value is not finite; both must start at zero (the
   // carved layout keeps the first 256 bytes for flags; the work counter is at
@@ -4049,13 +3303,14 @@ int search_dev_tc(const SearchArgs& a, cudaStream_t s) {
     if (timing) RBQ_CUDA(cudaEventRecord(ev[1], s));
     const int32_t* npq = a.per_query_nprobe ? a.per_query_nprobe + q0 : nullptr;
     if (a.pred) {
-      RBQ_CHECK(predict_chunk(a, Q, cd.as<float>(), nqc, q0, fid.as<int32_t>(),
-                              fdist.as<float>(), s));
+      // (a probe past a query's count has no bucket: -1 in the list)
+      RBQ_CUDA(cudaMemsetAsync(probe_ids, 0xff, sizeof(int32_t) * nqc * nprobe, s));
+      RBQ_CHECK(predict_chunk(a, Q, cd.as<float>(), nqc, nprobe, a.pred_nprobe + q0,
+                              fid.as<int32_t>(), fdist.as<float>(), probe_ids, probe_dist, s));
       npq = a.pred_nprobe + q0;
+    } else {
+      RBQ_CHECK(probe_select(X, Q, nqc, cd.as<float>(), nprobe, npq, probe_ids, probe_dist, s));
     }
-    RBQ_CHECK(probe_select(X, Q, nqc, cd.as<float>(), nprobe, npq, probe_ids, probe_dist, s,
-                           a.pred ? fid.as<int32_t>() : nullptr, fdist.as<float>(),
-                           std::min(kMlpIn, K)));
     if (metric_ip(X)) RBQ_CHECK(probe_nq2(X, Q, nqc, nprobe, probe_ids, pnq2.as<float>(), s));
     if (timing) RBQ_CUDA(cudaEventRecord(ev[2], s));
     float* rqp = a.trace && a.trace->rq ? a.trace->rq + q0 * dpad : rq.as<float>();

@@ -238,13 +238,18 @@ __device__ __forceinline__ int64_t tiled_off(int64_t r, int k, int R, int nks) {
 // padded matrix; column 0 also folds the norm.
 __global__ void pack_centroids_kernel(const float* __restrict__ C, int K, int d, int Kp,
                                       int64_t rows, float* __restrict__ ctf,
-                                      float* __restrict__ cn2, float* __restrict__ cnorm) {
+                                      float* __restrict__ cn2, float* __restrict__ cnorm,
+                                      float* __restrict__ rot) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= rows * Kp) return;
   const int64_t c = i / Kp;
   const int k = (int)(i % Kp);
   const float* row = C + c * d;
   ctf[tiled_off(c, k, kPdN, Kp / kPdEl)] = (c < K && k < d) ? to_tf32(row[k]) : 0.0f;
+  const int ld = (d + 31) / 32 * 32;  // (at most Kp)
+  if (c < K && k < ld)
+    rot[c * ld + (k & ~31) + ((((k >> 3) & 3) + (int)(c & 3)) & 3) * 8 + (k & 7)] =
+        k < d ? row[k] : 0.0f;
   if (k == 0 && c < K) {
     float s2 = 0.0f;
     for (int t = 0; t < d; ++t) s2 = __fmaf_rn(row[t], row[t], s2);
@@ -271,12 +276,18 @@ __global__ void max_norm_kernel(const float* __restrict__ cnorm, int K, float* _
 // One warp per query row (rows past M: zeros): the row rounded to TF32 in
 // tiles of kPdM rows, its FP32 ||q||^2 (lane-strided partial folds, then a
 // fixed butterfly; the bound needs an FP32 value of the norm, not the
-// canonical fold) and the initial range of its keys.
+// canonical fold) and the initial range of its keys; also clears the counts
+// of the selection's two redo lists.
 __global__ void query_prep_kernel(const float* __restrict__ Q, int64_t M, int d, int Kp,
                                   int64_t rows, float* __restrict__ qt, float* __restrict__ nq2,
-                                  uint32_t* __restrict__ kmin, uint32_t* __restrict__ kmax) {
+                                  uint32_t* __restrict__ kmin, uint32_t* __restrict__ kmax,
+                                  int* __restrict__ redo, int* __restrict__ redo_mlp) {
   const int64_t m = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  if (m == 0 && lane == 0) {
+    *redo = 0;
+    *redo_mlp = 0;
+  }
   if (m >= rows) return;
   const int nks = Kp / kPdEl;
   float part = 0.0f;
@@ -292,23 +303,6 @@ __global__ void query_prep_kernel(const float* __restrict__ Q, int64_t M, int d,
     kmin[m] = 0xffffffffu;
     kmax[m] = 0u;
   }
-}
-
-// Bounded wait that also gives up once another role of the CTA has failed.
-__device__ __forceinline__ bool pd_wait(uint32_t bar, uint32_t parity, volatile int* fail,
-                                        uint32_t limit = kWaitLimit) {
-  for (uint32_t it = 0; it < limit; ++it) {
-    uint32_t done;
-    asm volatile(
-        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (done) return true;
-    if ((it & 255) == 255 && *fail) return false;
-  }
-  return false;
 }
 
 // The products Qt Ct^T (M x N) over tiles (m, n), m-major, turned into the
@@ -651,6 +645,10 @@ ProbeScratch probe_scratch(const rabitq_index* X, int64_t nq, float* base) {
   v.pool_n = 2 * kProbePool * (int)((X->K + kPdN - 1) / kPdN);
   v.pool = reinterpret_cast<uint32_t*>(base + o);
   o = align_up(o + (size_t)nq * v.pool_n, 64);
+  v.redo = reinterpret_cast<int*>(base + o);
+  o = align_up(o + (size_t)nq + 1, 64);
+  v.redo_mlp = reinterpret_cast<int*>(base + o);
+  o = align_up(o + (size_t)nq + 1, 64);
   v.floats = o;
   return v;
 }
@@ -663,7 +661,7 @@ int pack_centroids(rabitq_index* X, cudaStream_t s) {
   const int64_t rows = centroid_tile_rows(X->K);
   const int64_t total = rows * X->kp;
   pack_centroids_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(
-      X->centroids, X->K, X->d, X->kp, rows, X->ctf, X->cn2, X->cnorm);
+      X->centroids, X->K, X->d, X->kp, rows, X->ctf, X->cn2, X->cnorm, X->cent_rot);
   RBQ_CUDA(cudaGetLastError());
   max_norm_kernel<<<1, 1024, 0, s>>>(X->cnorm, X->K, X->cnorm_max);
   RBQ_CUDA(cudaGetLastError());
@@ -676,8 +674,8 @@ int probe_keys_tc(const rabitq_index* X, const float* Q, int64_t M, float* scrat
   const int N = X->K, Kp = X->kp, nks = Kp / kPdEl;
   const int64_t rows = (M + kPdM - 1) / kPdM * kPdM;
   const ProbeScratch v = probe_scratch(X, M, scratch);
-  query_prep_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(Q, M, X->d, Kp, rows, v.qt,
-                                                                        v.nq2, v.kmin, v.kmax);
+  query_prep_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(
+      Q, M, X->d, Kp, rows, v.qt, v.nq2, v.kmin, v.kmax, v.redo, v.redo_mlp);
   RBQ_CUDA(cudaGetLastError());
   const int ntn = (N + kPdN - 1) / kPdN;
   const int64_t items = (rows / kPdM) * ntn;

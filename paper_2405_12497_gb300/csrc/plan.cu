@@ -37,6 +37,9 @@ void destroy(rabitq_plan* P) {
   for (auto& kv : P->graphs) cudaGraphExecDestroy(kv.second);
   P->graphs.clear();
   if (P->cap_stream) cudaStreamDestroy(P->cap_stream);
+  if (P->a.side) cudaStreamDestroy(P->a.side);
+  if (P->a.fork) cudaEventDestroy(P->a.fork);
+  if (P->a.join) cudaEventDestroy(P->a.join);
   for (auto& e : P->ev)
     if (e) cudaEventDestroy(e);
   cudaFree(P->scratch);
@@ -169,6 +172,9 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
     if (e == cudaSuccess) e = cudaMemset(P->scratch, 0, 256);  // the error flag
     if (e == cudaSuccess) e = cudaMemset(P->queries, 0, sizeof(float) * nq_max * X->d);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&a.side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&a.join, cudaEventDisableTiming);
     if (opts.collect_stats)
       for (auto& ev : P->ev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);

@@ -49,4 +49,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
   return false;
 }
 
+// Bounded wait that also gives up once another role of the CTA has failed.
+__device__ __forceinline__ bool pd_wait(uint32_t bar, uint32_t parity, volatile int* fail,
+                                        uint32_t limit = kWaitLimit) {
+  for (uint32_t it = 0; it < limit; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if ((it & 255) == 255 && *fail) return false;
+  }
+  return false;
+}
+
 }  // namespace rbq

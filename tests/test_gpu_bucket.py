@@ -1,0 +1,100 @@
+"""The bucket-major scan of large batches (kernels_bucket.cu) against the
+per-query scan (explicit CTA layout) and the oracle: ids and distance bits are
+equal. eps0 = 0 makes every bound the estimate itself, so that one wrong
+product changes which codes survive."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def R():
+    from paper_2405_12497_gb300 import rabitq
+    return rabitq
+
+
+def _mix(rng, n, d, comps=40):
+    mu = rng.standard_normal((comps, d))
+    return (mu[rng.integers(0, comps, n)] + 0.6 * rng.standard_normal((n, d))).astype(np.float32)
+
+
+def _same(R, G, Q, k, nprobe, **kw):
+    import torch
+    qd = torch.from_numpy(Q).cuda()
+    ids, dist = G.search(qd, k, nprobe, **kw)
+    ref_i, ref_d = G.search(qd, k, nprobe, layout=R.LAYOUT_CTA, staging=R.STAGING_OFF, **kw)
+    assert torch.equal(ids, ref_i)
+    assert torch.equal(dist.view(torch.int32), ref_d.view(torch.int32))
+    return ids.cpu().numpy(), dist.cpu().numpy()
+
+
+# code lengths: one operand stage, a half stage, several, the 16-pair items of
+# the longest; d below the code length (padding)
+@pytest.mark.parametrize("d,bits", [(50, 64), (128, 128), (100, 192), (256, 256), (300, 320),
+                                    (420, 448), (960, 1024), (2000, 2048), (4000, 4096)])
+def test_code_lengths(R, d, bits):
+    rng = np.random.default_rng(bits)
+    n = 9000 if d <= 512 else 3000
+    data, Q = _mix(rng, n, d), _mix(rng, 1000, d)
+    G = R.Index.build(data, 24, seed=2, code_bits=bits, kmeans_iters=3)
+    for k, nprobe, eps0 in ((10, 5, 0.0), (100, 7, 1.9), (1, 24, 0.5)):
+        _same(R, G, Q, k, nprobe, eps0=eps0)
+
+
+@pytest.mark.parametrize("metric", ["l2", "ip", "cosine"])
+@pytest.mark.parametrize("bq", [1, 3, 4])
+def test_metrics_and_bits(R, metric, bq):
+    rng = np.random.default_rng(7)
+    data, Q = _mix(rng, 8000, 128), _mix(rng, 1003, 128)
+    G = R.Index.build(data, 32, seed=2, kmeans_iters=3, metric=metric)
+    for k, nprobe in ((1, 3), (20, 9), (256, 32)):
+        _same(R, G, Q, k, nprobe, bq=bq)
+        _same(R, G, Q, k, nprobe, bq=bq, eps0=0.0)
+
+
+# batch and bucket edges: 1000 is the smallest batch; K = 1 is one bucket of
+# many tiles and several items, K = 1000 buckets of three codes with a few
+# pairs each (fewer than k codes probed: pads), 1031 odd
+@pytest.mark.parametrize("nq,K,nprobe,k", [(1000, 16, 4, 10), (1031, 1, 1, 100),
+                                           (1031, 1000, 16, 64), (1000, 3, 3, 256),
+                                           (2000, 700, 2, 10)])
+def test_batch_edges_match_the_oracle(R, oracle_mod, nq, K, nprobe, k):
+    from paper_2405_12497_gb300 import synth
+    data, Q = synth.tiny(n=3000, nq=nq)
+    G = R.Index.build(data, K, seed=2, kmeans_iters=3)
+    ids, dist = _same(R, G, Q, k, nprobe)
+    O = oracle_mod.OracleIndex(data, K=K, seed=2, iters=3)
+    m = min(nq, 120)
+    ids_o, dist_o = O.search(Q[:m], k, nprobe)
+    assert np.array_equal(ids[:m], ids_o)
+    assert np.array_equal(dist[:m].view(np.uint32), dist_o.view(np.uint32))
+
+
+def test_ties_counts_and_plans(R):
+    """Identical points (every bound equal), per-query probe counts, and a
+    plan's replay, once below the batch rule."""
+    import torch
+    rng = np.random.default_rng(3)
+    data = np.repeat(_mix(rng, 40, 128), 150, axis=0)
+    Q = _mix(rng, 1100, 128)
+    G = R.Index.build(data, 20, seed=2, kmeans_iters=3)
+    _same(R, G, Q, 100, 6)
+    npq = torch.from_numpy(rng.integers(1, 12, 1100).astype(np.int32)).cuda()
+    _same(R, G, Q, 30, 11, per_query_nprobe=npq)
+    plan = R.Plan(G, 100, 6, 1100)
+    ids, dist = G.search(Q, 100, 6, layout=R.LAYOUT_CTA)
+    for nq in (1100, 90, 1000):
+        i, x = plan.search(Q[:nq])
+        assert np.array_equal(i, ids[:nq]) and np.array_equal(x.view(np.uint32),
+                                                              dist[:nq].view(np.uint32))
+
+
+def test_long_lists_are_redone(R):
+    """A bound so wide that every code of 16k-code buckets is a candidate: the
+    lists (8192 entries for k <= 32) overflow and the per-query scan takes
+    those queries."""
+    rng = np.random.default_rng(5)
+    data, Q = _mix(rng, 33000, 64, comps=2), _mix(rng, 1000, 64, comps=2)
+    G = R.Index.build(data, 2, seed=2, kmeans_iters=2)
+    _same(R, G, Q, 10, 1, eps0=40.0)
