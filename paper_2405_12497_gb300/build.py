@@ -16,8 +16,9 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "librabitq.so")
 BUILD_DIR = os.path.join(HERE, "_build")
 SOURCES = [
-    "api.cu", "api_predictor.cu", "kernels_gemm.cu", "kernels_build.cu", "kernels_search.cu", "kernels_bucket.cu",
-    "kernels_tc.cu", "kernels_mlp.cu", "noalloc.cu", "plan.cu", "shard.cu",
+    "api.cu", "api_predictor.cu", "kernels_gemm.cu", "kernels_build.cu", "kernels_assign.cu",
+    "kernels_search.cu", "kernels_bucket.cu", "kernels_tc.cu",
+    "kernels_mlp.cu", "noalloc.cu", "plan.cu", "shard.cu",
     "server.cu",
 ]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -255,8 +255,19 @@ int rabitq_build(const float* data, int64_t n, int32_t d, int32_t n_clusters, ui
     RBQ_CHECK(transpose_f32(X->centroids, n_clusters, d, X->centroids_t, s));
     RBQ_CHECK(pack_centroids(X, s));
     RBQ_CHECK(adist.alloc(sizeof(float) * n, s));
-    RBQ_CHECK(argmin_sqdist(ddata, d, X->centroids_t, n_clusters, n, n_clusters, d, X->assign,
-                            adist.as<float>(), s));
+    {
+      AssignWork w;  // without room for its scratch: the canonical tiles
+      const bool tc = assign_tc_applies(n, n_clusters) && w.alloc(n, d, n_clusters, s) == RABITQ_OK;
+      cudaGetLastError();
+      if (tc) {
+        RBQ_CHECK(assign_rows(ddata, X->centroids, X->centroids_t, n, n_clusters, d, w, X->assign,
+                              adist.as<float>(), s));
+        RBQ_CHECK(w.check(s));
+      } else {
+        RBQ_CHECK(argmin_sqdist(ddata, d, X->centroids_t, n_clusters, n, n_clusters, d, X->assign,
+                                adist.as<float>(), s));
+      }
+    }
     RBQ_CHECK(counting_sort(X->assign, n, n_clusters, X->perm, X->bucket_off, s));
     RBQ_CHECK(invert_perm(X->perm, n, X->inv_perm, s));
     RBQ_CHECK(gather_rows_f32(ddata, d, X->perm, n, d, X->data_b, s));

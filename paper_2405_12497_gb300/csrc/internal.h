@@ -141,6 +141,27 @@ int gemm_canon(GemmOp op, const float* A, int64_t lda, const int32_t* a_rows, co
 // argmin_n of squared distance rows (ties to the lower n): assign[m], dist[m]
 int argmin_sqdist(const float* A, int64_t lda, const float* Bt, int64_t ldb, int64_t M, int N,
                   int K, int32_t* assign, float* dist, cudaStream_t s);
+// the rows of a device list (its count, at most M, then the rows), unless
+// there are `most` or fewer
+int argmin_sqdist_list(const float* A, int64_t lda, const float* Bt, int64_t ldb, int64_t M, int N,
+                       int K, const int32_t* list, int most, int32_t* assign, float* dist,
+                       cudaStream_t s);
+
+// ---- tensor-core k-means assignment (kernels_assign.cu) ------------------
+// argmin_sqdist's results for packed rows (lda = d) against K centroids, C
+// and its transpose Ct. The scratch is made for one set of rows: the calls
+// that share it pass the same A and M, with any C.
+struct AssignWork {
+  DevBuf ct, vec, xt, top, redo;
+  int nks = 0, ntn = 0, parts = 0;
+  int64_t chunk = 0;
+  bool ready = false;  // mu and, in one chunk, the rows' tiles are made
+  int alloc(int64_t M, int d, int K, cudaStream_t s);
+  int check(cudaStream_t s);  // after the last call: a wait that expired
+};
+bool assign_tc_applies(int64_t M, int K);
+int assign_rows(const float* A, const float* C, const float* Ct, int64_t M, int K, int d,
+                AssignWork& w, int32_t* assign, float* dist, cudaStream_t s);
 
 // ---- build (kernels_build.cu) -------------------------------------------
 int exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaStream_t s);

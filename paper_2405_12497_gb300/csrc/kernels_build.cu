@@ -653,15 +653,22 @@ int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters
   RBQ_CHECK(a.alloc(sizeof(int32_t) * m, s));
   RBQ_CHECK(perm.alloc(sizeof(int32_t) * m, s));
   RBQ_CHECK(off.alloc(sizeof(int32_t) * (K + 1), s));
+  AssignWork w;  // without room for its scratch: the canonical tiles
+  const bool tc = iters > 0 && assign_tc_applies(m, K) && w.alloc(m, d, K, s) == RABITQ_OK;
+  cudaGetLastError();
   for (int it = 0; it < iters; ++it) {
     RBQ_CHECK(transpose_f32(centroids, K, d, ct.as<float>(), s));
-    RBQ_CHECK(argmin_sqdist(train, d, ct.as<float>(), K, m, K, d, a.as<int32_t>(), nullptr, s));
+    if (tc)
+      RBQ_CHECK(assign_rows(train, centroids, ct.as<float>(), m, K, d, w, a.as<int32_t>(), nullptr,
+                            s));
+    else
+      RBQ_CHECK(argmin_sqdist(train, d, ct.as<float>(), K, m, K, d, a.as<int32_t>(), nullptr, s));
     RBQ_CHECK(counting_sort(a.as<int32_t>(), m, K, perm.as<int32_t>(), off.as<int32_t>(), s));
     kmeans_update_kernel<<<K, 128, 0, s>>>(train, d, perm.as<int32_t>(), off.as<int32_t>(),
                                           centroids);
     RBQ_CUDA(cudaGetLastError());
   }
-  return RABITQ_OK;
+  return tc ? w.check(s) : RABITQ_OK;
 }
 
 int encode_dev(rabitq_index* X, const float* adist_b, cudaStream_t s) {

@@ -177,19 +177,25 @@ __global__ void __launch_bounds__(256) rows_canon_kernel(const float* __restrict
 }
 
 // Row-wise argmin of canonical squared distances, ties to the lower column.
+// With a list (its count, then rows): those rows, if there are more than `most`.
 __global__ void __launch_bounds__(NT) argmin_sqdist_kernel(const float* __restrict__ A,
                                                            int64_t lda,
                                                            const float* __restrict__ Bt,
                                                            int64_t ldb, int64_t M, int N, int K,
-                                                           int32_t* __restrict__ assign,
+                                                           const int32_t* __restrict__ list,
+                                                           int most, int32_t* __restrict__ assign,
                                                            float* __restrict__ dist) {
   __shared__ float As[BK][BM];
   __shared__ float Bs[BK][BN];
   const int64_t m0 = (int64_t)blockIdx.x * BM;
+  if (list) {
+    M = *list++;
+    if (M <= most || m0 >= M) return;
+  }
   const float* arow[4];
   const float* srow[4];
   bool aval[4];
-  row_pointers<false>(A, lda, nullptr, nullptr, 0, nullptr, m0, M, arow, srow, aval);
+  row_pointers<false>(A, lda, list, nullptr, 0, nullptr, m0, M, arow, srow, aval);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float best[8];
   int bidx[8];
@@ -233,8 +239,9 @@ __global__ void __launch_bounds__(NT) argmin_sqdist_kernel(const float* __restri
     for (int i = 0; i < 8; ++i) {
       const int64_t gm = m0 + ty + 16 * i;
       if (gm < M) {
-        assign[gm] = (bidx[i] == 0x7fffffff) ? 0 : bidx[i];  // all-infinite row
-        if (dist) dist[gm] = best[i];
+        const int64_t row = list ? list[gm] : gm;
+        assign[row] = (bidx[i] == 0x7fffffff) ? 0 : bidx[i];  // all-infinite row
+        if (dist) dist[row] = best[i];
       }
     }
   }
@@ -278,7 +285,17 @@ int argmin_sqdist(const float* A, int64_t lda, const float* Bt, int64_t ldb, int
                   int K, int32_t* assign, float* dist, cudaStream_t s) {
   if (M <= 0) return RABITQ_OK;
   dim3 grid((unsigned)((M + BM - 1) / BM));
-  argmin_sqdist_kernel<<<grid, NT, 0, s>>>(A, lda, Bt, ldb, M, N, K, assign, dist);
+  argmin_sqdist_kernel<<<grid, NT, 0, s>>>(A, lda, Bt, ldb, M, N, K, nullptr, 0, assign, dist);
+  RBQ_CUDA(cudaGetLastError());
+  return RABITQ_OK;
+}
+
+int argmin_sqdist_list(const float* A, int64_t lda, const float* Bt, int64_t ldb, int64_t M, int N,
+                       int K, const int32_t* list, int most, int32_t* assign, float* dist,
+                       cudaStream_t s) {
+  if (M <= most) return RABITQ_OK;
+  dim3 grid((unsigned)((M + BM - 1) / BM));
+  argmin_sqdist_kernel<<<grid, NT, 0, s>>>(A, lda, Bt, ldb, M, N, K, list, most, assign, dist);
   RBQ_CUDA(cudaGetLastError());
   return RABITQ_OK;
 }
