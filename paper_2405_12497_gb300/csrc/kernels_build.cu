@@ -256,42 +256,117 @@ __global__ void gaussian_kernel(uint64_t seed, int64_t pairs, double* __restrict
   G[2 * m + 1] = g1;
 }
 
-// Gram-Schmidt, one projection pass of row i: c_j = <v, p_j> for j < i
-// (PT is P transposed so that threads j read consecutive addresses).
-__global__ void gs_dot_kernel(const double* __restrict__ v, const double* __restrict__ PT, int i,
-                              int dpad, double* __restrict__ c) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= i) return;
-  double s = 0.0;
-  for (int k = 0; k < dpad; ++k) s = __fma_rn(v[k], PT[(int64_t)k * dpad + j], s);
-  c[j] = s;
-}
+// Gram-Schmidt with two projection passes per row, every sum a chain in
+// ascending order: c_j = <v, p_j> for j < i; v_k -= sum_{j<i} c_j p_j[k];
+// the same again; p_i = v / ||v||. One cooperative launch: CTA b owns the
+// rows and columns 32 b .. 32 b + 31, a lane of its first warp one of each
+// (one warp a CTA: more CTAs, fewer rows to read for each); v and c pass through global memory between grid
+// barriers, five per row. The chains bound it: 3 to 5 dpad dependent FMAs a
+// row, whose operands come from shared memory (v, c) and from registers
+// loaded 32 steps ahead (P). A dependent FP64 FMA takes 64 cycles here
+// whatever the number of lanes, which makes 140 ms of the 1024 rows of 1024
+// (measured: 184; with a launch per phase and a load in every step 353), and
+// 128 rows of 128 take 4.4 ms (11.5).
+constexpr int kGsThreads = 256, kGsAhead = 32;
 
-// v_k -= sum_{j<i} c_j p_j[k]
-__global__ void gs_update_kernel(double* __restrict__ v, const double* __restrict__ P,
-                                 const double* __restrict__ c, int i, int dpad) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= dpad) return;
-  double t = 0.0;
-  for (int j = 0; j < i; ++j) t = __fma_rn(c[j], P[(int64_t)j * dpad + k], t);
-  v[k] = __dsub_rn(v[k], t);
-}
-
-// p_i = v / ||v||; also writes the transposed copy. One block of dpad threads
-// (dpad <= 1024 is enforced by the caller via the grid-stride loop).
-__global__ void gs_normalize_kernel(const double* __restrict__ v, int i, int dpad,
-                                    double* __restrict__ P, double* __restrict__ PT) {
-  __shared__ double nrm;
+__device__ __forceinline__ bool gs_barrier(unsigned* bar, unsigned target, int* err) {
+  __shared__ int s_ok;
+  __syncthreads();
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int k = 0; k < dpad; ++k) s = __fma_rn(v[k], v[k], s);
-    nrm = __dsqrt_rn(s);
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    int ok = 0;
+    for (int it = 0; it < (1 << 21) && !ok; ++it) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      ok = (int)(v - target) >= 0;
+    }
+    if (!ok) atomicExch(err, 1);
+    s_ok = ok;
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < dpad; k += blockDim.x) {
-    const double p = __ddiv_rn(v[k], nrm);
-    P[(int64_t)i * dpad + k] = p;
-    PT[(int64_t)k * dpad + i] = p;
+  return s_ok != 0;
+}
+
+__device__ __forceinline__ void gs_load(double (&x)[kGsAhead], const double* __restrict__ p,
+                                        int64_t ld, int n) {
+#pragma unroll
+  for (int u = 0; u < kGsAhead; ++u)
+    if (u < n) x[u] = __ldcg(p + u * ld);
+}
+
+// fold of f[t] * p[t ld], t < n ascending; x holds the first group
+__device__ __forceinline__ double gs_fold(const double* __restrict__ f,
+                                          const double* __restrict__ p, int64_t ld, int n,
+                                          double (&x)[kGsAhead]) {
+  double s = 0.0;
+  int t = 0;
+  for (; t + kGsAhead <= n; t += kGsAhead) {
+    double y[kGsAhead];
+    gs_load(y, p + (t + kGsAhead) * ld, ld, n - t - kGsAhead);
+#pragma unroll
+    for (int u = 0; u < kGsAhead; ++u) s = __fma_rn(f[t + u], x[u], s);
+#pragma unroll
+    for (int u = 0; u < kGsAhead; ++u) x[u] = y[u];
+  }
+#pragma unroll
+  for (int u = 0; u < kGsAhead; ++u)
+    if (t + u < n) s = __fma_rn(f[t + u], x[u], s);
+  return s;
+}
+
+__global__ void __launch_bounds__(kGsThreads, 1) gram_schmidt_kernel(
+    const double* __restrict__ G, int dpad, double* P, double* PT, double* v, double* c,
+    unsigned* bar, int* err) {
+  extern __shared__ __align__(16) double gs_row[];  // the staged v or c
+  __shared__ double s_norm;
+  const int o = blockIdx.x * 32 + threadIdx.x;  // the lane's row and column
+  const bool lane = threadIdx.x < 32;
+  unsigned done = 0;
+  double x[kGsAhead];
+  auto meet = [&]() { return gs_barrier(bar, done += gridDim.x, err); };
+  auto stage = [&](const double* src, int n) {
+    for (int t0 = threadIdx.x; t0 < n; t0 += 4 * kGsThreads) {
+      double y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t0 + u * kGsThreads < n) y[u] = __ldcg(src + t0 + u * kGsThreads);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t0 + u * kGsThreads < n) gs_row[t0 + u * kGsThreads] = y[u];
+    }
+    __syncthreads();
+  };
+  for (int i = 0; i < dpad; ++i) {
+    const double* g = G + (int64_t)i * dpad;
+    const bool dots = lane && o < i;
+    double vk = lane ? __ldcg(g + o) : 0.0;
+    for (int pass = 0; pass < 2 && i > 0; ++pass) {
+      if (dots) gs_load(x, PT + o, dpad, dpad);
+      stage(pass ? v : g, dpad);
+      if (dots) c[o] = gs_fold(gs_row, PT + o, dpad, dpad, x);
+      if (lane) gs_load(x, P + o, dpad, i);
+      if (!meet()) return;
+      stage(c, i);
+      if (lane) {
+        vk = __dsub_rn(vk, gs_fold(gs_row, P + o, dpad, i, x));
+        v[o] = vk;
+      }
+      if (!meet()) return;
+    }
+    stage(i > 0 ? v : g, dpad);
+    if (threadIdx.x == 0) {
+      double s = 0.0;
+#pragma unroll 16
+      for (int k = 0; k < dpad; ++k) s = __fma_rn(gs_row[k], gs_row[k], s);
+      s_norm = __dsqrt_rn(s);
+    }
+    __syncthreads();
+    if (lane) {
+      const double p = __ddiv_rn(vk, s_norm);
+      P[(int64_t)i * dpad + o] = p;
+      PT[(int64_t)o * dpad + i] = p;
+    }
+    if (!meet()) return;
   }
 }
 
@@ -316,45 +391,67 @@ __global__ void compact_kernel(const int32_t* __restrict__ flags, const int32_t*
   if (i < n && flags[i]) ids[pos[i]] = (int32_t)i;
 }
 
-// Floyd's sampling of K distinct indices of [0, m), in the order chosen.
-// Sequential by nature (each pick depends on the set so far); K <= 65536.
+// Floyd's sampling of K distinct indices of [0, m), in the order chosen (2048
+// of 400k: 0.91 ms one draw at a time, 0.08 so):
+// pick t is r_t, a draw from [0, m - K + t], or m - K + t if r_t is taken. Each
+// pick depends on the set so far, so one warp takes 32 draws at a time: their
+// marks are loaded together, the picks among the 32 settled in registers.
 __global__ void floyd_kernel(int64_t m, int K, uint64_t seed, uint8_t* __restrict__ taken,
                              int32_t* __restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int t = 0; t < K; ++t) {
+  const int lane = threadIdx.x;
+  for (int t0 = 0; t0 < K; t0 += 32) {
+    const int t = t0 + lane;
+    const bool live = t < K;
     const unsigned long long j = (unsigned long long)(m - K + t);
     const U4 w = philox4x32_10(seed, (uint32_t)t, 0u, 0u, kTagKmeansInit);
-    const unsigned long long r = ((unsigned long long)w.x * (j + 1)) >> 32;
-    const unsigned long long pick = taken[r] ? j : r;
-    taken[pick] = 1;
-    out[t] = (int32_t)pick;
+    const int r = live ? (int)(((unsigned long long)w.x * (j + 1)) >> 32) : -1;
+    bool hit = live && taken[r];
+    int pick = hit ? (int)j : r;
+    // earlier draws of the 32, final in ascending order, may take r
+    for (int u = 0; u < 31; ++u) {
+      const int pu = __shfl_sync(kFull, pick, u);
+      if (lane > u && pu == r) pick = (int)j;
+    }
+    if (live) {
+      taken[pick] = 1;
+      out[t] = pick;
+    }
+    __syncwarp();
   }
 }
 
 // Mean update: centroid c = (sum of its members in ascending id order) /
-// count; an empty cluster keeps its centroid.
-__global__ void kmeans_update_kernel(const float* __restrict__ x, int d,
-                                     const int32_t* __restrict__ perm,
-                                     const int32_t* __restrict__ off,
-                                     float* __restrict__ centroids) {
-  const int c = blockIdx.x;
+// count; an empty cluster keeps its centroid. A block takes a cluster and 128
+// dimensions. The chain over the members bounds it (a large cluster's most),
+// so its loads run kUpAhead members ahead (32 ahead: slower, the remainder goes
+// in fours). 400k x 128, 2048 clusters: 260 to 155 us with 4 and 16 ahead;
+// 50k x 960, 512 clusters: 1.77 to 0.33 ms with the dimensions in blocks.
+constexpr int kUpAhead = 16;
+__global__ void __launch_bounds__(128) kmeans_update_kernel(const float* __restrict__ x, int d,
+                                                            const int32_t* __restrict__ perm,
+                                                            const int32_t* __restrict__ off,
+                                                            float* __restrict__ centroids) {
+  const int c = blockIdx.x, i = blockIdx.y * 128 + threadIdx.x;
   const int beg = off[c], end = off[c + 1];
-  if (end == beg) return;
-  const float cnt = __int2float_rn(end - beg);
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
-    float s = 0.0f;
-    int p = beg;
-    for (; p + 4 <= end; p += 4) {  // loads issued ahead; adds stay in order
-      const float a0 = x[(int64_t)perm[p] * d + i], a1 = x[(int64_t)perm[p + 1] * d + i];
-      const float a2 = x[(int64_t)perm[p + 2] * d + i], a3 = x[(int64_t)perm[p + 3] * d + i];
-      s = __fadd_rn(s, a0);
-      s = __fadd_rn(s, a1);
-      s = __fadd_rn(s, a2);
-      s = __fadd_rn(s, a3);
-    }
-    for (; p < end; ++p) s = __fadd_rn(s, x[(int64_t)perm[p] * d + i]);
-    centroids[(int64_t)c * d + i] = __fdiv_rn(s, cnt);
+  if (end == beg || i >= d) return;
+  float s = 0.0f;
+  int p = beg;
+  for (; p + kUpAhead <= end; p += kUpAhead) {
+    float a[kUpAhead];
+#pragma unroll
+    for (int u = 0; u < kUpAhead; ++u) a[u] = __ldg(x + (int64_t)__ldg(perm + p + u) * d + i);
+#pragma unroll
+    for (int u = 0; u < kUpAhead; ++u) s = __fadd_rn(s, a[u]);
   }
+  for (; p + 4 <= end; p += 4) {
+    float a[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] = __ldg(x + (int64_t)__ldg(perm + p + u) * d + i);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s = __fadd_rn(s, a[u]);
+  }
+  for (; p < end; ++p) s = __fadd_rn(s, x[(int64_t)perm[p] * d + i]);
+  centroids[(int64_t)c * d + i] = __fdiv_rn(s, __int2float_rn(end - beg));
 }
 
 // ------------------------------------------------------------ encoding
@@ -588,29 +685,27 @@ int check_finite(const float* x, int64_t count, cudaStream_t s, bool* finite) {
 
 int sample_rotation_dev(uint64_t seed, int32_t dpad, double* P64, float* P32, cudaStream_t s) {
   const int64_t total = (int64_t)dpad * dpad;
-  DevBuf G, PT, v, c;
+  DevBuf G, PT, v;
   RBQ_CHECK(G.alloc(sizeof(double) * total, s));
   RBQ_CHECK(PT.alloc(sizeof(double) * total, s));
-  RBQ_CHECK(v.alloc(sizeof(double) * dpad, s));
-  RBQ_CHECK(c.alloc(sizeof(double) * dpad, s));
+  RBQ_CHECK(v.alloc(sizeof(double) * 2 * dpad + 16, s));  // v, c, barrier, error
   gaussian_kernel<<<blocks_for(total / 2, 128), 128, 0, s>>>(seed, total / 2, G.as<double>());
   RBQ_CUDA(cudaGetLastError());
-  for (int i = 0; i < dpad; ++i) {
-    RBQ_CUDA(cudaMemcpyAsync(v.p, G.as<double>() + (int64_t)i * dpad, sizeof(double) * dpad,
-                             cudaMemcpyDeviceToDevice, s));
-    if (i > 0) {
-      for (int pass = 0; pass < 2; ++pass) {
-        gs_dot_kernel<<<blocks_for(i, 64), 64, 0, s>>>(v.as<double>(), PT.as<double>(), i, dpad,
-                                                      c.as<double>());
-        gs_update_kernel<<<blocks_for(dpad, 64), 64, 0, s>>>(v.as<double>(), P64, c.as<double>(),
-                                                            i, dpad);
-      }
-    }
-    gs_normalize_kernel<<<1, 256, 0, s>>>(v.as<double>(), i, dpad, P64, PT.as<double>());
-  }
-  RBQ_CUDA(cudaGetLastError());
+  const double* g = G.as<double>();
+  double *pt = PT.as<double>(), *vp = v.as<double>(), *c = vp + dpad;
+  unsigned* bar = reinterpret_cast<unsigned*>(c + dpad);
+  int* err = reinterpret_cast<int*>(bar + 1);
+  RBQ_CUDA(cudaMemsetAsync(bar, 0, 16, s));
+  void* args[] = {&g, &dpad, &P64, &pt, &vp, &c, &bar, &err};
+  // dpad / 32 <= 128 CTAs
+  RBQ_CUDA(cudaLaunchCooperativeKernel((const void*)gram_schmidt_kernel, dim3(dpad / 32),
+                                       dim3(kGsThreads), args, sizeof(double) * dpad, s));
   to_f32_kernel<<<blocks_for(total, 256), 256, 0, s>>>(P64, total, P32);
   RBQ_CUDA(cudaGetLastError());
+  int h_err = 0;
+  RBQ_CUDA(cudaMemcpyAsync(&h_err, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+  RBQ_CUDA(cudaStreamSynchronize(s));
+  if (h_err) return fail(RABITQ_ETIMEOUT, "a grid barrier expired in the rotation's sampling");
   return RABITQ_OK;
 }
 
@@ -664,7 +759,7 @@ int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters
     else
       RBQ_CHECK(argmin_sqdist(train, d, ct.as<float>(), K, m, K, d, a.as<int32_t>(), nullptr, s));
     RBQ_CHECK(counting_sort(a.as<int32_t>(), m, K, perm.as<int32_t>(), off.as<int32_t>(), s));
-    kmeans_update_kernel<<<K, 128, 0, s>>>(train, d, perm.as<int32_t>(), off.as<int32_t>(),
+    kmeans_update_kernel<<<dim3(K, (d + 127) / 128), 128, 0, s>>>(train, d, perm.as<int32_t>(), off.as<int32_t>(),
                                           centroids);
     RBQ_CUDA(cudaGetLastError());
   }
