@@ -161,6 +161,12 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
   if (st == RABITQ_OK) {
     P->bytes = carved_bytes(a, P->grid, nq_max);
     e = cudaMalloc(reinterpret_cast<void**>(&P->scratch), P->bytes);
+    if (e == cudaErrorMemoryAllocation && a.allow_bucket) {  // the smaller per-query scratch
+      cudaGetLastError();
+      a.allow_bucket = 0;
+      P->bytes = carved_bytes(a, P->grid, nq_max);
+      e = cudaMalloc(reinterpret_cast<void**>(&P->scratch), P->bytes);
+    }
     if (e == cudaSuccess)
       e = cudaMalloc(reinterpret_cast<void**>(&P->queries), sizeof(float) * nq_max * X->d);
     if (e == cudaSuccess)
