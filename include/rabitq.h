@@ -66,7 +66,9 @@ enum { RABITQ_SCAN_AUTO = 0, RABITQ_SCAN_POPC = 1, RABITQ_SCAN_TC = 2 };
  * per query (no block barriers; D' of 128 or 256, B_q = 4, k <= 128 and
  * batches large enough to fill the GPU; other searches use the CTA layout).
  * AUTO follows rabitq_autotune's choice, else the warp layout where it
- * applies. Results are identical in every layout. */
+ * applies; batches of 1000 queries and more (B_q <= 4, k <= 256, no trace, four
+ * probes and more per bucket) it scans bucket by bucket on the tensor cores.
+ * Results are identical in every layout. */
 enum { RABITQ_LAYOUT_AUTO = 0, RABITQ_LAYOUT_CTA = 1, RABITQ_LAYOUT_WARP = 2 };
 
 /* Staging of the CTA layout's scan rounds (D' of 128 or 256, B_q = 4): each
