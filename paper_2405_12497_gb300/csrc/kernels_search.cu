@@ -2757,7 +2757,8 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
   RBQ_CHECK(rq.alloc(sizeof(float) * qchunk * dpad, s));
   RBQ_CHECK(pid.alloc(sizeof(int32_t) * qchunk * nprobe, s));
   RBQ_CHECK(pdist.alloc(sizeof(float) * qchunk * nprobe, s));
-  RBQ_CHECK(cand.alloc(sizeof(int4) * std::max<int64_t>(grid, qchunk * split) * a.cand_cap, s));
+  RBQ_CHECK(cand.alloc(sizeof(int4) * (split > 1 ? std::max<int64_t>(grid, qchunk * split) : grid) *
+                           a.cand_cap, s));  // a list per resident CTA
   RBQ_CHECK(err.alloc(sizeof(int), s));
   if (split > 1) {
     RBQ_CHECK(ubout.alloc(sizeof(uint32_t) * qchunk * split * a.k, s));
