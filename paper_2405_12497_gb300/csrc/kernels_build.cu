@@ -259,9 +259,9 @@ __global__ void gaussian_kernel(uint64_t seed, int64_t pairs, double* __restrict
 // Gram-Schmidt with two projection passes per row, every sum a chain in
 // ascending order: c_j = <v, p_j> for j < i; v_k -= sum_{j<i} c_j p_j[k];
 // the same again; p_i = v / ||v||. One cooperative launch: CTA b owns the
-// rows and columns 32 b .. 32 b + 31, a lane of its first warp one of each
-// (one warp a CTA: more CTAs, fewer rows to read for each); v and c pass through global memory between grid
-// barriers, five per row. The chains bound it: 3 to 5 dpad dependent FMAs a
+// rows and columns 32 b .. 32 b + 31 (the last CTA those below dpad), a lane of
+// its first warp one of each (one warp a CTA: more CTAs, fewer rows to read for
+// each); v and c pass through global memory between grid barriers, five per row. The chains bound it: 3 to 5 dpad dependent FMAs a
 // row, whose operands come from shared memory (v, c) and from registers
 // loaded 32 steps ahead (P). A dependent FP64 FMA takes 64 cycles here
 // whatever the number of lanes, which makes 140 ms of the 1024 rows of 1024
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kGsThreads, 1) gram_schmidt_kernel(
   extern __shared__ __align__(16) double gs_row[];  // the staged v or c
   __shared__ double s_norm;
   const int o = blockIdx.x * 32 + threadIdx.x;  // the lane's row and column
-  const bool lane = threadIdx.x < 32;
+  const bool lane = threadIdx.x < 32 && o < dpad;
   unsigned done = 0;
   double x[kGsAhead];
   auto meet = [&]() { return gs_barrier(bar, done += gridDim.x, err); };
@@ -697,8 +697,8 @@ int sample_rotation_dev(uint64_t seed, int32_t dpad, double* P64, float* P32, cu
   int* err = reinterpret_cast<int*>(bar + 1);
   RBQ_CUDA(cudaMemsetAsync(bar, 0, 16, s));
   void* args[] = {&g, &dpad, &P64, &pt, &vp, &c, &bar, &err};
-  // dpad / 32 <= 128 CTAs
-  RBQ_CUDA(cudaLaunchCooperativeKernel((const void*)gram_schmidt_kernel, dim3(dpad / 32),
+  // at most 128 CTAs (dpad <= 4096, any even size)
+  RBQ_CUDA(cudaLaunchCooperativeKernel((const void*)gram_schmidt_kernel, dim3((dpad + 31) / 32),
                                        dim3(kGsThreads), args, sizeof(double) * dpad, s));
   to_f32_kernel<<<blocks_for(total, 256), 256, 0, s>>>(P64, total, P32);
   RBQ_CUDA(cudaGetLastError());

@@ -41,6 +41,15 @@ def test_rotation_bit_exact(R, oracle_mod, dpad):
     assert np.abs(P @ P.T - np.eye(dpad)).max() <= 1e-13
 
 
+# every even size is accepted: below one block of 32 columns, with a part of a
+# block at the end, and whole blocks that are no multiple of 64
+@pytest.mark.parametrize("dpad", [2, 30, 32, 34, 48, 96, 100, 130, 1000])
+def test_rotation_sizes_off_the_block(R, oracle_mod, dpad):
+    P = R.sample_rotation(5, dpad)
+    Po = oracle_mod.sample_rotation(5, dpad)
+    assert np.array_equal(P.view(np.uint64), Po.view(np.uint64))
+
+
 def test_build_bit_exact(R, oracle_mod, tiny_gpu_index, tiny_oracle_index):
     G, O = tiny_gpu_index, tiny_oracle_index
     assert (G.n, G.d, G.dpad, G.K) == (O.n, O.d, O.dpad, O.K)
