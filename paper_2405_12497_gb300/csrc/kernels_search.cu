@@ -150,6 +150,16 @@ __device__ void select_row(F score, int K, int nsel, int nprobe, int sort_n,
 // within d 2^-23 ||q|| ||c|| and (d + 2) 2^-24 (||q|| + ||c||)^2 of exact,
 // and the FP32 operations forming s~, U and L add a few units of
 // 2^-24 (||q|| + ||c||)^2; eps_c takes all of these with a 5% margin.
+//
+// All of this needs the squared norms in range (probe_bounded): past 2^62 the
+// sum of two of them, or eps_c, may overflow while the canonical score of the
+// nearest centroid does not, and of a query that is not finite there is no
+// bound at all. The row select ranks every centroid of such a query. Every
+// entry of a list is written in any case: later kernels use the ids as
+// addresses.
+__device__ __forceinline__ bool probe_bounded(float nq, float nc_max) {
+  return __fadd_rn(nq, nc_max) < 0x1.0p62f;  // (false for a NaN)
+}
 constexpr int kProbeCandMax = 2048;  // candidates kept in shared memory
 
 __global__ void __launch_bounds__(kThreads) probe_select_kernel(
@@ -190,7 +200,22 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
     s_pmin = 0xffffffffu;
     s_pmax = 0u;
   }
-  const ProbeEps eps(metric, __fsqrt_rn(nq2_q[q]), d);
+  int32_t* oid = out_ids + (int64_t)q * nprobe;
+  float* od = out_dist + (int64_t)q * nprobe;
+  auto select_all = [&]() {  // the row select over canonical scores computed on
+    select_row(              // the fly (every pass refolds them; a rare path)
+        [qs, C, ld, metric](int c) {
+          return metric ? row_score_rot<true>(C, c, qs, ld) : row_score_rot<false>(C, c, qs, ld);
+        },
+        K, nsel, nprobe, sort_n, reinterpret_cast<unsigned long long*>(work), oid, od);
+  };
+  const float nq = __fsqrt_rn(nq2_q[q]);
+  if (!probe_bounded(nq, __ldg(cnorm_max))) {
+    __syncthreads();  // (the query is staged)
+    select_all();
+    continue;
+  }
+  const ProbeEps eps(metric, nq, d);
   constexpr int kSelU = 8;  // keys per thread in flight in a pass
   int* hist = reinterpret_cast<int*>(work);
   for (int i = tid; i < kHistBins; i += blockDim.x) hist[i] = 0;
@@ -368,9 +393,7 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
   }
   __syncthreads();
   const int nc = s_nc;
-  int32_t* oid = out_ids + (int64_t)q * nprobe;
-  float* od = out_dist + (int64_t)q * nprobe;
-  if (nc <= kProbeCandMax) {
+  if (nc >= nsel && nc <= kProbeCandMax) {  // (fewer than nsel: no list has holes)
     // canonical scores of the candidates (one thread each, the full scan's
     // fold); every line of their rows is requested first
     for (int i = tid; i < nc; i += blockDim.x) {
@@ -405,13 +428,7 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
       od[j] = __int_as_float(0x7f800000);
     }
   } else {
-    // too many candidates: the row select over canonical scores computed on
-    // the fly (every pass refolds them; a rare path)
-    select_row(
-        [qs, C, ld, metric](int c) {
-          return metric ? row_score_rot<true>(C, c, qs, ld) : row_score_rot<false>(C, c, qs, ld);
-        },
-        K, nsel, nprobe, sort_n, reinterpret_cast<unsigned long long*>(work), oid, od);
+    select_all();  // too many candidates
   }
   }
 }
@@ -420,9 +437,9 @@ __global__ void __launch_bounds__(kThreads) probe_select_kernel(
 // between its short steps, and as many queries in flight per SM as warps (a
 // CTA per query waited at some fifteen barriers for little work). 62 of 4096,
 // 10k queries: 84 us against 133; 16 of 1024, 8000 queries: 27 against 76.
-// The threshold comes from a histogram of kWarpBins bins; a query with more
-// than kWarpCand candidates goes to redo (count, then the queries) for the
-// CTA kernel.
+// The threshold comes from a histogram of kWarpBins bins; a query without
+// bounds or with more than kWarpCand candidates goes to redo (count, then the
+// queries) for the CTA kernel.
 constexpr int kPsWarps = 4, kWarpBins = 256, kWarpCand = 512;
 __global__ void __launch_bounds__(32 * kPsWarps) probe_select_warp_kernel(
     const float* __restrict__ Q, int64_t nq, int d, const uint32_t* __restrict__ keys,
@@ -451,7 +468,12 @@ __global__ void __launch_bounds__(32 * kPsWarps) probe_select_warp_kernel(
   nsel = min(nsel, K);
   for (int i = lane; i < ld; i += 32) qs[i] = i < d ? __ldg(Q + q * d + i) : 0.0f;
   for (int i = lane; i < kWarpBins; i += 32) hist[i] = 0;
-  const ProbeEps eps(metric, __fsqrt_rn(nq2_q[q]), d);
+  const float nqn = __fsqrt_rn(nq2_q[q]);
+  if (!probe_bounded(nqn, __ldg(cnorm_max))) {
+    if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int)q;
+    return;
+  }
+  const ProbeEps eps(metric, nqn, d);
   int cnt = 0;
   uint32_t pmin = 0xffffffffu, pmax = 0u;
   for (int i = lane; i < pool_n; i += 32) {
@@ -582,7 +604,7 @@ __global__ void __launch_bounds__(32 * kPsWarps) probe_select_warp_kernel(
   } else {
     consider_run(0, K);
   }
-  if (nc > kWarpCand) {
+  if (nc < nsel || nc > kWarpCand) {
     if (lane == 0) redo[1 + atomicAdd(redo, 1)] = (int)q;
     return;
   }

@@ -98,3 +98,32 @@ def test_long_lists_are_redone(R):
     data, Q = _mix(rng, 33000, 64, comps=2), _mix(rng, 1000, 64, comps=2)
     G = R.Index.build(data, 2, seed=2, kmeans_iters=2)
     _same(R, G, Q, 10, 1, eps0=40.0)
+
+
+# a query whose squared norm overflows (every distance infinite: the lowest
+# ids), one near the limit and one with a NaN, among ordinary ones; probe lists
+# by a warp per query and, above 64 probes, by a CTA
+@pytest.mark.parametrize("nprobe", [9, 70])
+def test_overflowing_queries_leave_the_batch_alone(R, oracle_mod, nprobe):
+    from paper_2405_12497_gb300 import synth
+    data, Q = synth.tiny(n=6000, nq=1100)
+    Q = Q.copy()
+    unit = Q / np.linalg.norm(Q, axis=1, keepdims=True)
+    Q[7], Q[300], Q[1099] = unit[7] * 1e20, unit[300] * 4e18, unit[1099] * 3e17
+    G = R.Index.build(data, 100, seed=2, kmeans_iters=3)
+    ids, dist = _same(R, G, Q, 10, nprobe)
+    O = oracle_mod.OracleIndex(data, K=100, seed=2, iters=3)
+    rows = [*range(60), 300, *range(1050, 1100)]
+    for i in rows:  # (the quantization stream is the query's index in the call)
+        t = O.trace(Q[i], i, 10, nprobe)
+        assert np.array_equal(ids[i], t["ids"]), i
+        assert np.array_equal(dist[i].view(np.uint32), t["dist"].view(np.uint32)), i
+    bad = Q.copy()
+    bad[500, 3] = np.nan
+    with pytest.raises(Exception, match="non-finite"):
+        G.search(bad, 10, nprobe)
+    plan = R.Plan(G, 10, nprobe, 1100)
+    pi, pd = plan.search(bad)
+    ok = np.arange(1100) != 500
+    assert np.array_equal(pi[ok], ids[ok])
+    assert np.array_equal(pd[ok].view(np.uint32), dist[ok].view(np.uint32))

@@ -51,6 +51,20 @@ def test_probe_lists_match_full_scan(R, oracle_mod, d, K, scale, nprobe):
     _check(R, oracle_mod, data, cents, Q, nprobe)
 
 
+def test_probe_lists_where_squared_norms_overflow(R, oracle_mod):
+    """||q||^2 + ||c||^2 overflows FP32 while the nearest centroids' distances do
+    not: the filter has no bound, every centroid is ranked canonically."""
+    rng = np.random.default_rng(23)
+    d, K = 24, 300
+    cents = rng.standard_normal((K, d))
+    cents = (cents / np.linalg.norm(cents, axis=1, keepdims=True) * 1.5e19).astype(np.float32)
+    data = (cents * (1 + 1e-3 * rng.standard_normal((K, d)))).astype(np.float32)
+    Q = (cents[:24] * (1 + 1e-2 * rng.standard_normal((24, d)))).astype(np.float32)
+    Q[5] *= 10                   # ||q||^2 itself overflows
+    _check(R, oracle_mod, data, cents, Q, 20)
+    _check(R, oracle_mod, data, cents, Q, 200)
+
+
 def test_crowded_group_is_scanned_in_full(R, oracle_mod):
     """The 64 nearest centroids of some queries have ids 0..63 (one group of
     128 centroids): that group's 8 pooled keys are all under the threshold,
