@@ -11,7 +11,8 @@
 //                           first codes (nearest probes): tau0 >= tau_ub
 //   2. bucket_count / bucket_plan / bucket_quant: (query, probe) pairs
 //                           grouped by bucket, quantized (§3.3.1) into
-//                           operand rows; work items {bucket, pairs, codes}
+//                           operand rows; work items {bucket, pairs, codes};
+//                           the room a query's candidate list may take
 //   3. bucket_scan<1>       every code: upper bounds <= tau0, per query;
 //      bucket_tau_kernel    tau_ub, the k-th smallest of them (exact)
 //   4. bucket_scan<2>       every code again: the candidates LB <= tau_ub
@@ -22,7 +23,12 @@
 // exact, the estimator is evaluated in the same FP32 order, and the re-rank
 // rule depends on the candidate set only, not on the order it was found in.
 // A query whose candidate list outgrows its capacity goes to the redo list,
-// which the per-query kernel runs.
+// which the per-query kernel runs, a CTA for each: some milliseconds for a
+// query of 256 large buckets, however few they are. So the lists share one
+// pool, and where most queries probe few codes (learned counts) the others get
+// room for several times the even share (13 of 10k queries of a learned batch,
+// 10M x 256, had up to 54k candidates against a share of 32k: 6.29 ms with
+// them redone, 4.66 all per query, 3.68 so).
 //
 // Measured (GB300, order to re-rank of one batch, per-query kernel -> this):
 //   10k queries x 62 probes, 1M x 128, K 4096, k 100        4.83 -> 2.47 ms
@@ -59,6 +65,7 @@ constexpr int kGTilesPerItem = 4;        // code tiles per work item
 constexpr int kGPad = 16;                // a bucket's pair slots start at a multiple of this
 constexpr int kGTau0Probes = 16;         // probes the first threshold may look at
 constexpr float kGSlack = 0x1.0p-18f;    // prefilter slack (bucket_scan_kernel)
+constexpr int kGLevels = 6;              // list capacities: the even share << level
 
 struct BucketParams {
   const uint64_t* codes;
@@ -76,9 +83,10 @@ struct BucketParams {
   const int32_t* sq;         // pair slots: query
   const float* tau;          // queries: the pass's threshold
   uint32_t* ulist;           // pass 1: queries x capu upper-bound keys
-  int4* list;                // pass 2: queries x capl {position, LB, estimate, UB}
+  int4* list;                // pass 2: the lists {position, LB, estimate, UB}
+  const int2* lrow;          // pass 2: queries: a list's first entry and capacity
   int* cnt;                  // queries: hits of this pass
-  int cap;
+  int cap;                   // pass 1
   int* err;
 };
 
@@ -138,14 +146,33 @@ __device__ __forceinline__ int probes_of(const FusedParams& P, int64_t q) {
   return P.nprobe_q ? min(max(P.nprobe_q[q], 1), P.nprobe) : P.nprobe;
 }
 
-// One warp per query (learned counts are mostly far below nprobe).
-__global__ void bucket_count_kernel(FusedParams P, int32_t* __restrict__ bcnt) {
+// One warp per query (learned counts are mostly far below nprobe). Also the
+// entries that all candidate lists would take at each level of capacity
+// (share << level, and never more than the query's codes): lsum.
+__global__ void __launch_bounds__(256) bucket_count_kernel(FusedParams P, int share,
+                                                           int32_t* __restrict__ bcnt,
+                                                           unsigned long long* __restrict__ lsum) {
+  __shared__ int s_codes[8];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (q >= P.nq) return;
-  const int np = probes_of(P, q);
-  for (int j = threadIdx.x & 31; j < np; j += 32) {
-    const int c = P.probe_ids[q * P.nprobe + j];
-    if (c >= 0) atomicAdd(bcnt + c, 1);
+  int codes = 0;
+  if (q < P.nq) {
+    const int np = probes_of(P, q);
+    for (int j = lane; j < np; j += 32) {
+      const int c = P.probe_ids[q * P.nprobe + j];
+      if (c >= 0) {
+        atomicAdd(bcnt + c, 1);
+        codes += __ldg(P.bucket_off + c + 1) - __ldg(P.bucket_off + c);
+      }
+    }
+  }
+  codes = __reduce_add_sync(kFull, codes);
+  if (lane == 0) s_codes[wid] = codes;
+  __syncthreads();
+  if (threadIdx.x < kGLevels) {
+    unsigned long long sum = 0;
+    for (int w = 0; w < 8; ++w) sum += min((int64_t)s_codes[w], (int64_t)share << threadIdx.x);
+    atomicAdd(lsum + threadIdx.x, sum);
   }
 }
 
@@ -351,20 +378,27 @@ __global__ void __launch_bounds__(256) bucket_quant_kernel(FusedParams P,
 }
 
 // ---------------------------------------------------------- first threshold
+struct ListPool {
+  const unsigned long long* sum;  // kGLevels (bucket_count_kernel)
+  unsigned* used;
+  unsigned size;                  // entries (below 2^31)
+  int share;
+};
+
 // tau0 of a query: the k-th smallest upper bound of its first `want` codes
 // (in probe order, at most kGTau0Probes probes), +inf when there are fewer
 // than k. The k-th smallest of any subset bounds tau_ub from above. Of a
 // query with at most want_max codes all are looked at: that is tau_ub itself,
 // and tau0 = -inf keeps pass 1 from the query. Also clears the query's hit
-// counters. One CTA per query.
+// counters and takes its candidate list from the pool, at the highest level at
+// which all lists fit (level 0 does: the pool has a share for each). One CTA
+// per query.
 // (The CTA is short steps that wait on each other: the CTAs resident set the
 // rate, so registers are held to what six -- four for longer codes -- allow.)
 template <int WT, int BQT>
-__global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(FusedParams P, int want_max,
-                                                               float* __restrict__ tau0,
-                                                               float* __restrict__ taub,
-                                                               int* __restrict__ ucnt,
-                                                               int* __restrict__ lcnt) {
+__global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
+    FusedParams P, int want_max, ListPool lp, float* __restrict__ tau0, float* __restrict__ taub,
+    int* __restrict__ ucnt, int* __restrict__ lcnt, int2* __restrict__ lrow) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ SelState s_sel;
   __shared__ float4 s_meta[kGTau0Probes];
@@ -416,6 +450,10 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
   if (tid == 0) {
     ucnt[q] = 0;
     lcnt[q] = 0;
+    int l = kGLevels - 1;
+    while (l > 0 && lp.sum[l] > lp.size) --l;
+    const int cap = (int)min((int64_t)codes, (int64_t)lp.share << l);
+    lrow[q] = make_int2((int)atomicAdd(lp.used, (unsigned)cap), cap);
   }
   __syncthreads();
   const int m = s_np;
@@ -519,6 +557,7 @@ struct __align__(16) ColMeta {
   float4 ex[kGN];              // A, B, E, add
   float2 pt[kGN];              // sum(q_u), tau
   int q[kGN];
+  int2 lr[kGN];                // pass 2: lrow
 };
 
 __host__ __device__ inline size_t bucket_smem_bytes(int nt, int dpad) {
@@ -593,6 +632,7 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
       float4 m[kGN / 32];
       float ps[kGN / 32], tau[kGN / 32];
       int q[kGN / 32];
+      int2 lr[kGN / 32];
 #pragma unroll
       for (int u = 0; u < kGN / 32; ++u) {
         const int j = u * 32 + lane;
@@ -606,8 +646,11 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
         }
       }
 #pragma unroll
-      for (int u = 0; u < kGN / 32; ++u)
-        tau[u] = x.c >= 0 && u * 32 + lane < x.cols ? __ldg(P.tau + q[u]) : __int_as_float(0xff800000);
+      for (int u = 0; u < kGN / 32; ++u) {
+        const bool in = x.c >= 0 && u * 32 + lane < x.cols;
+        tau[u] = in ? __ldg(P.tau + q[u]) : __int_as_float(0xff800000);
+        if (MODE == 2) lr[u] = in ? __ldg(P.lrow + q[u]) : make_int2(0, 0);
+      }
       if (MODE == 1 && x.c >= 0) {  // an item whose queries all know their tau_ub
         float best = tau[0];
 #pragma unroll
@@ -634,6 +677,7 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
         M.ex[j] = m[u];
         M.pt[j] = make_float2(ps[u], tau[u]);
         M.q[j] = q[u];
+        if (MODE == 2) M.lr[j] = lr[u];
         const float xmax = m[u].x * ps[u] + fabsf(m[u].y) * (float)P.dpad;
         float* pre = reinterpret_cast<float*>(M.pre[j >> 1]) + (j & 1);
         pre[0] = m[u].x;
@@ -792,9 +836,11 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
           for (int i0 = 0; __any_sync(kFull, i0 < n); i0 += 4) {
             float lb[4], est[4], ub[4];
             int qq[4], slot[4];
+            int2 lr[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               qq[u] = -1;
+              lr[u] = make_int2(0, P.cap);
               lb[u] = est[u] = ub[u] = 0.0f;
               if (i0 + u < n) {
                 const uint32_t e = queue[(i0 + u) * 32];
@@ -812,7 +858,10 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
                   qq[u] = M.q[col];
                   lb[u] = bound;
                   est[u] = dist;
-                  if (MODE == 2) ub[u] = __fadd_rn(dist, er);
+                  if (MODE == 2) {
+                    ub[u] = __fadd_rn(dist, er);
+                    lr[u] = M.lr[col];
+                  }
                 }
               }
             }
@@ -820,13 +869,13 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
             for (int u = 0; u < 4; ++u) slot[u] = qq[u] >= 0 ? atomicAdd(P.cnt + qq[u], 1) : 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-              if (qq[u] >= 0 && slot[u] < P.cap) {
-                const int64_t at = (int64_t)qq[u] * P.cap + slot[u];
+              if (qq[u] >= 0 && slot[u] < lr[u].y) {
                 if (MODE == 1)
-                  P.ulist[at] = float_key(lb[u]);
+                  P.ulist[(int64_t)qq[u] * P.cap + slot[u]] = float_key(lb[u]);
                 else
-                  P.list[at] = make_int4(pos, __float_as_int(lb[u]), __float_as_int(est[u]),
-                                         __float_as_int(ub[u]));
+                  P.list[lr[u].x + slot[u]] = make_int4(pos, __float_as_int(lb[u]),
+                                                        __float_as_int(est[u]),
+                                                        __float_as_int(ub[u]));
               }
             }
           }
@@ -1060,9 +1109,9 @@ constexpr int kTailKeys = 4096;  // estimate keys kept in shared memory
 
 struct TailParams {
   FusedParams P;
-  int4* list;            // queries x capl {position, LB, estimate, UB}
+  int4* list;            // {position, LB, estimate, UB}
   const int* lcnt;
-  int capl;
+  const int2* lrow;      // a query's first entry and capacity
   const int* ucnt;
   int capu;
   const float* taub;
@@ -1115,11 +1164,12 @@ __global__ void __launch_bounds__(kThreads, 4) bucket_tail_kernel(TailParams T) 
     const int64_t q = s_q;
     if (q >= P.nq) break;
     int n = T.lcnt[q];
-    if (n > T.capl) {
+    const int2 lr = T.lrow[q];
+    if (n > lr.y) {
       if (tid == 0) P.redo[atomicAdd(P.redo_cnt, 1)] = (int32_t)q;
       continue;
     }
-    int4* L = T.list + q * T.capl;
+    int4* L = T.list + lr.x;
     for (int i = tid; i < d; i += kThreads) qv[i] = P.queries[q * d + i];
     QueryBounds B;
     if (T.qrec) {
@@ -1144,7 +1194,7 @@ __global__ void __launch_bounds__(kThreads, 4) bucket_tail_kernel(TailParams T) 
       }));
       if (tid == 0) s_cnt = n;
       __syncthreads();  // (compact_cand reads the count first)
-      compact_cand(L, &s_cnt, T.capl, s_scratch,
+      compact_cand(L, &s_cnt, lr.y, s_scratch,
                    [tau_ub](const int4& e) { return __int_as_float(e.y) <= tau_ub; });
       n = s_cnt;
     }
@@ -1343,7 +1393,7 @@ size_t tail_smem_bytes(int ct, int ce, int sk, int d) {
          align_up(sizeof(float) * d, 16) + 32 * (size_t)((d + 15) / 16);
 }
 
-typedef void (*Tau0Fn)(FusedParams, int, float*, float*, int*, int*);
+typedef void (*Tau0Fn)(FusedParams, int, ListPool, float*, float*, int*, int*, int2*);
 Tau0Fn pick_tau0(int W, int bq) {
   if (bq == 4) {
     if (W == 2) return bucket_tau0_kernel<2, 4>;
@@ -1353,10 +1403,15 @@ Tau0Fn pick_tau0(int W, int bq) {
   return bucket_tau0_kernel<0, 0>;
 }
 
-// Codes the first threshold looks at, and the capacities of the two lists.
+// Codes the first threshold looks at, the capacity of the upper-bound lists and
+// the even share of the candidate lists' pool.
 int tau0_codes(int k) { return std::min(4096, std::max(512, 10 * k)) + 15 & ~15; }
 int cap_upper(int k) { return k <= 32 ? 4096 : 8192; }
-int cap_cand(int k) { return k <= 32 ? 8192 : 32768; }
+int list_share(const SearchArgs& a) {
+  const int64_t codes = std::min<int64_t>(
+      a.X->n, (int64_t)std::min(a.nprobe, a.X->K) * std::max(a.X->max_bucket, 1));
+  return (int)std::min<int64_t>(a.k <= 32 ? 8192 : 32768, codes);
+}
 
 int pairs_per_item(int dpad) {
   return std::max(kGPad, std::min(kGN, 32768 / dpad / kGPad * kGPad));
@@ -1365,13 +1420,16 @@ int pairs_per_item(int dpad) {
 struct BucketScratch {
   int32_t *bcnt, *bfill, *boff;
   int4* items;
-  int* ctl;  // [0] items, [32] [64] work counters of the passes, [96] tail counter
+  // [0] items, [16] the levels' sums (64-bit), [32] [64] work counters of the
+  // passes, [96] tail counter, [112] pool entries taken
+  int* ctl;
   uint8_t* qop;
   float4* smeta;
   float* spsum;
   int32_t* sq;
   float *tau0, *taub;
   int *ucnt, *lcnt;
+  int2* lrow;
   uint32_t* ulist;
   int4* list;
   int* redo;  // [0] count, [32] the redo launch's work counter, list from [64]
@@ -1408,8 +1466,9 @@ BucketScratch bucket_carve(const SearchArgs& a, int64_t nq, unsigned char* base)
   b.taub = reinterpret_cast<float*>(take(sizeof(float) * nq));
   b.ucnt = reinterpret_cast<int*>(take(sizeof(int) * nq));
   b.lcnt = reinterpret_cast<int*>(take(sizeof(int) * nq));
+  b.lrow = reinterpret_cast<int2*>(take(sizeof(int2) * nq));
   b.ulist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * nq * cap_upper(a.k)));
-  b.list = reinterpret_cast<int4*>(take(sizeof(int4) * nq * cap_cand(a.k)));
+  b.list = reinterpret_cast<int4*>(take(sizeof(int4) * nq * list_share(a)));
   b.qrec = take((size_t)nq * query_stride(X->d));
   b.bytes = o;
   return b;
@@ -1418,7 +1477,7 @@ BucketScratch bucket_carve(const SearchArgs& a, int64_t nq, unsigned char* base)
 // Most queries scanned together: bounds the lists and the operand rows to
 // about 6 and 2 GiB.
 int64_t bucket_batch(const SearchArgs& a) {
-  const int64_t lists = (int64_t)cap_cand(a.k) * 16 + (int64_t)cap_upper(a.k) * 4;
+  const int64_t lists = (int64_t)list_share(a) * 16 + (int64_t)cap_upper(a.k) * 4;
   const int64_t rows = (int64_t)std::min(a.nprobe, a.X->K) * (a.X->dpad + 32);
   return std::max<int64_t>(1, std::min((int64_t(6) << 30) / lists, (int64_t(2) << 30) / rows));
 }
@@ -1465,7 +1524,7 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
   const int64_t per = (P0.nq + nb - 1) / nb;
   const BucketScratch b = bucket_carve(a, per, scratch);
   const int K = X->K, nt = pairs_per_item(X->dpad), want = tau0_codes(a.k);
-  const int capu = cap_upper(a.k), capl = cap_cand(a.k);
+  const int capu = cap_upper(a.k), share = list_share(a);
   int dev = 0, sms = 0, optin = 0;
   RBQ_CUDA(cudaGetDevice(&dev));
   RBQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1507,11 +1566,17 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
     P.out_dist += q0 * P.k;
     P.order = nullptr;
     RBQ_CUDA(cudaMemsetAsync(b.bcnt, 0, sizeof(int32_t) * (2 * K + 192), s));  // counts, ctl, redo
-    bucket_count_kernel<<<blocks(P.nq * 32, 256), 256, 0, s>>>(P, b.bcnt);
+    ListPool lp;
+    lp.sum = reinterpret_cast<unsigned long long*>(b.ctl + 16);
+    lp.used = reinterpret_cast<unsigned*>(b.ctl + 112);
+    lp.size = (unsigned)(per * share);
+    lp.share = share;
+    bucket_count_kernel<<<blocks(P.nq * 32, 256), 256, 0, s>>>(
+        P, share, b.bcnt, reinterpret_cast<unsigned long long*>(b.ctl + 16));
     bucket_plan_kernel<<<1, 1024, 0, s>>>(b.bcnt, X->bucket_off, K, nt, b.boff, b.items, b.ctl);
     bucket_quant_kernel<<<blocks(P.nq * quant_runs(P.nprobe) * 32, 256), 256, 0, s>>>(
         P, b.boff, b.bfill, b.qop, b.smeta, b.spsum, b.sq);
-    t0<<<(unsigned)P.nq, kThreads, t0_smem, s>>>(P, want, b.tau0, b.taub, b.ucnt, b.lcnt);
+    t0<<<(unsigned)P.nq, kThreads, t0_smem, s>>>(P, want, lp, b.tau0, b.taub, b.ucnt, b.lcnt, b.lrow);
     RBQ_CUDA(cudaGetLastError());
     BucketParams B;
     B.codes = X->codes;
@@ -1531,6 +1596,7 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
     B.err = P.err;
     B.ulist = b.ulist;
     B.list = b.list;
+    B.lrow = b.lrow;
     B.work = b.ctl + 32;
     B.tau = b.tau0;
     B.cnt = b.ucnt;
@@ -1541,7 +1607,6 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
     B.work = b.ctl + 64;
     B.tau = b.taub;
     B.cnt = b.lcnt;
-    B.cap = capl;
     bucket_scan_kernel<2><<<(unsigned)(2 * sms), kGThreads, scan_smem, s>>>(B);
     RBQ_CUDA(cudaGetLastError());
     if (T.qrec)
@@ -1554,7 +1619,7 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
     T.P.redo_cnt = b.redo;
     T.list = b.list;
     T.lcnt = b.lcnt;
-    T.capl = capl;
+    T.lrow = b.lrow;
     T.ucnt = b.ucnt;
     T.capu = capu;
     T.taub = b.taub;
