@@ -444,6 +444,15 @@ int rabitq_autotune_tiles(rabitq_index* idx, const float* queries, int64_t nq, i
  * into a CUDA graph; later runs replay it. Results equal rabitq_search's
  * with scan_path RABITQ_SCAN_POPC. The index and predictor must outlive the
  * plan. Errors: those of rabitq_search's arguments; EUNSUPPORTED; ENOMEM.
+ *
+ * Device memory of a large batch (RABITQ_LAYOUT_AUTO): the bucket-major scan
+ * takes, per query, 16 bytes for each of min(32768, the codes of nprobe largest
+ * buckets) list entries (8192 for k <= 32), 32 KB (16 KB) of upper bounds and
+ * about nprobe (D' + 36) bytes, at most 8 GiB in all: 5.2 GiB for 10k queries at
+ * k = 100. A search takes it from the device's default memory pool, which keeps
+ * it for later searches; a plan holds it. Where it, or anything allocated with
+ * it, does not fit, the per-query scan runs, whose scratch does not grow with
+ * the list entries (0.6 GB at 65536 max_candidates).
  */
 int rabitq_plan_create(const rabitq_index* idx, const rabitq_predictor* pr, int64_t nq_max,
                        int32_t k, int32_t nprobe, int32_t bq, float eps0,

@@ -2724,7 +2724,9 @@ int search_dev(const SearchArgs& a_in, cudaStream_t s) {
   return search_dev_popc(a, s);
 }
 
-int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
+namespace {
+
+int search_popc_run(const SearchArgs& a, bool* by_bucket_out, cudaStream_t s) {
   const rabitq_index* X = a.X;
   const int K = X->K, d = X->d, dpad = X->dpad, W = X->W;
   const int nprobe = std::min(a.nprobe, K);
@@ -2755,15 +2757,10 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
   if (wfn) RBQ_CHECK(warp_ctas(wfn, &wctas));
   const int capw = warp_capw(a);
   DevBuf candw, redo, wkey, worder, wooff, wsortws;
-  // the bucket-major scan, where it applies (without memory for its lists the
-  // per-query scan runs)
-  const bool bucket = split == 1 && bucket_applies(a, std::min(qchunk, a.nq));
+  const bool by_bucket = split == 1 && bucket_applies(a, std::min(qchunk, a.nq));
+  *by_bucket_out = by_bucket;
   DevBuf bscratch;
-  const bool by_bucket = bucket && bscratch.alloc(bucket_bytes(a, qchunk), s) == RABITQ_OK;
-  if (bucket && !by_bucket) {
-    cudaGetLastError();
-    set_error("");
-  }
+  if (by_bucket) RBQ_CHECK(bscratch.alloc(bucket_bytes(a, qchunk), s));
   if (wfn && !by_bucket) {
     RBQ_CHECK(candw.alloc(sizeof(int4) * wctas * (kWarpThreads / 32) * capw, s));
     RBQ_CHECK(redo.alloc(sizeof(int32_t) * (qchunk + 64), s));
@@ -2953,6 +2950,21 @@ int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
     return fail(RABITQ_EOVERFLOW,
                 "a query's candidate list exceeded max_candidates; raise max_candidates");
   return RABITQ_OK;
+}
+
+}  // namespace
+
+// The bucket-major scan, where it applies; where its lists or anything after
+// them find no memory, the per-query scan, which needs less.
+int search_dev_popc(const SearchArgs& a, cudaStream_t s) {
+  bool by_bucket = false;
+  const int st = search_popc_run(a, &by_bucket, s);
+  if (st != RABITQ_ENOMEM || !by_bucket) return st;
+  cudaGetLastError();
+  set_error("");
+  SearchArgs b = a;
+  b.allow_bucket = 0;
+  return search_popc_run(b, &by_bucket, s);
 }
 
 // ---------------------------------------------- carved (allocation-free) path

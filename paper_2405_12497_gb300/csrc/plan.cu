@@ -33,6 +33,18 @@ struct rabitq_plan {
 
 namespace {
 
+void free_buffers(rabitq_plan* P) {
+  cudaFree(P->scratch);
+  cudaFree(P->queries);
+  cudaFree(P->ids);
+  cudaFree(P->dist);
+  cudaFree(P->nprobe);
+  P->scratch = nullptr;
+  P->queries = P->dist = nullptr;
+  P->ids = nullptr;
+  P->nprobe = nullptr;
+}
+
 void destroy(rabitq_plan* P) {
   for (auto& kv : P->graphs) cudaGraphExecDestroy(kv.second);
   P->graphs.clear();
@@ -42,11 +54,7 @@ void destroy(rabitq_plan* P) {
   if (P->a.join) cudaEventDestroy(P->a.join);
   for (auto& e : P->ev)
     if (e) cudaEventDestroy(e);
-  cudaFree(P->scratch);
-  cudaFree(P->queries);
-  cudaFree(P->ids);
-  cudaFree(P->dist);
-  cudaFree(P->nprobe);
+  free_buffers(P);
   delete P;
 }
 
@@ -159,22 +167,24 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
   P->grid = grid;
   cudaError_t e = cudaSuccess;
   if (st == RABITQ_OK) {
-    P->bytes = carved_bytes(a, P->grid, nq_max);
-    e = cudaMalloc(reinterpret_cast<void**>(&P->scratch), P->bytes);
-    if (e == cudaErrorMemoryAllocation && a.allow_bucket) {  // the smaller per-query scratch
+    auto take = [&](void* pp, size_t bytes) {
+      if (e == cudaSuccess) e = cudaMalloc(static_cast<void**>(pp), bytes);
+    };
+    for (;;) {
+      e = cudaSuccess;
+      P->bytes = carved_bytes(a, P->grid, nq_max);
+      take(&P->scratch, P->bytes);
+      take(&P->queries, sizeof(float) * nq_max * X->d);
+      take(&P->ids, sizeof(int64_t) * nq_max * k);
+      take(&P->dist, sizeof(float) * nq_max * k);
+      if (pr) take(&P->nprobe, sizeof(int32_t) * nq_max);
+      if (e != cudaErrorMemoryAllocation || !a.allow_bucket) break;
+      // whichever did not fit: all of it once more with the smaller scratch of
+      // the per-query scan
       cudaGetLastError();
       a.allow_bucket = 0;
-      P->bytes = carved_bytes(a, P->grid, nq_max);
-      e = cudaMalloc(reinterpret_cast<void**>(&P->scratch), P->bytes);
+      free_buffers(P);
     }
-    if (e == cudaSuccess)
-      e = cudaMalloc(reinterpret_cast<void**>(&P->queries), sizeof(float) * nq_max * X->d);
-    if (e == cudaSuccess)
-      e = cudaMalloc(reinterpret_cast<void**>(&P->ids), sizeof(int64_t) * nq_max * k);
-    if (e == cudaSuccess)
-      e = cudaMalloc(reinterpret_cast<void**>(&P->dist), sizeof(float) * nq_max * k);
-    if (e == cudaSuccess && pr)
-      e = cudaMalloc(reinterpret_cast<void**>(&P->nprobe), sizeof(int32_t) * nq_max);
     if (e == cudaSuccess) e = cudaMemset(P->scratch, 0, 256);  // the error flag
     if (e == cudaSuccess) e = cudaMemset(P->queries, 0, sizeof(float) * nq_max * X->d);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking);
