@@ -67,7 +67,8 @@ enum { RABITQ_SCAN_AUTO = 0, RABITQ_SCAN_POPC = 1, RABITQ_SCAN_TC = 2 };
  * batches large enough to fill the GPU; other searches use the CTA layout).
  * AUTO follows rabitq_autotune's choice, else the warp layout where it
  * applies; batches of 1000 queries and more (B_q <= 4, k <= 256, no trace, four
- * probes and more per bucket) it scans bucket by bucket on the tensor cores.
+ * probes and more per bucket, enough codes for the further launches to pay) it
+ * scans bucket by bucket on the tensor cores.
  * Results are identical in every layout. */
 enum { RABITQ_LAYOUT_AUTO = 0, RABITQ_LAYOUT_CTA = 1, RABITQ_LAYOUT_WARP = 2 };
 

@@ -12,6 +12,12 @@
 
 using namespace rbq;
 
+float rabitq_predictor::mean_nprobe() const {
+  if (mean_at.empty()) return std::max(1.0f, (float)nprobe_max / 8.0f);
+  const float i = std::round(128.0f + 32.0f * std::log2(mult));
+  return mean_at[(size_t)std::min(std::max(i, 0.0f), (float)mean_at.size() - 1.0f)];
+}
+
 namespace {
 
 bool device_ptr(const void* p) {

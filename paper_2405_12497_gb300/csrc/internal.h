@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <vector>
 
 #include "../../include/rabitq.h"
 
@@ -70,6 +71,10 @@ struct rabitq_predictor {
   int64_t n_train = 0, n_val = 0;
   float* params = nullptr;  // RABITQ_MLP_PARAMS, BF16 values stored as FP32
   void* params_bf16 = nullptr;  // the same values packed as BF16 (inference)
+  // mean probe count of the validation queries at the multipliers 2^((i - 128)
+  // / 32) of the calibration (empty for a predictor made from parameters)
+  std::vector<float> mean_at;
+  float mean_nprobe() const;    // at mult; nprobe_max / 8 where it is not known
 };
 
 namespace rbq {
@@ -277,6 +282,9 @@ struct SearchArgs {
   // large batches may take the bucket-major scan (kernels_bucket.cu); off where
   // the scratch is fixed
   int allow_bucket = 1;
+  // probes per query that are expected: nprobe, or the predictor's mean at the
+  // multiplier it had when the call or plan was made (expect_probes)
+  float mean_probes = 0.0f;
   // bulk-copy staging of the CTA layout's scan rounds (RABITQ_STAGING_*;
   // AUTO resolves to the tuned or default choice)
   int32_t stage = 0;
@@ -312,8 +320,10 @@ int search_enqueue_carved(const SearchArgs& a, unsigned char* scratch, size_t sc
 size_t carved_bytes(const SearchArgs& a, int64_t grid, int64_t nq_max);
 // ---- bucket-major scan of large batches (kernels_bucket.cu)
 struct FusedParams;
-// whether a batch of nq queries takes it (an AUTO layout, many pairs per bucket)
+// whether a batch of nq queries takes it (an AUTO layout, enough work in all
+// and per bucket)
 bool bucket_applies(const SearchArgs& a, int64_t nq);
+void expect_probes(SearchArgs& a);
 size_t bucket_bytes(const SearchArgs& a, int64_t nq);
 int pack_rows(rabitq_index* X, cudaStream_t s);
 int bucket_search(const SearchArgs& a, const FusedParams& P, unsigned char* scratch,

@@ -1503,12 +1503,26 @@ int pack_rows(rabitq_index* X, cudaStream_t s) {
 bool bucket_applies(const SearchArgs& a, int64_t nq) {
   if (!a.allow_bucket || a.trace || a.bq > 4 || a.k > 256 || a.cand_cap < 65536) return false;
   if (a.layout != RABITQ_LAYOUT_AUTO || a.stage == RABITQ_STAGING_BULK) return false;
-  const int nprobe = std::min(a.nprobe, a.X->K);
-  const int64_t pairs = nq * (a.pred ? std::max(1, nprobe / 8) : nprobe);
-  // Below about four pairs per bucket the tiles are mostly padding, and below
-  // a thousand queries the re-rank kernel's last wave is mostly idle (777
-  // inner-product queries: 0.69 ms against 0.40 ms per query).
-  return nq >= 1000 && pairs >= 4 * (int64_t)a.X->K;
+  // Measured against the per-query scan on eight indexes (100k x 96 to 2M x 256,
+  // D' 128 to 1024, L2 and inner products), k 1 to 256, 320 to 10k queries, 4 to
+  // 128 probes. Below about four pairs per bucket the tiles are mostly padding.
+  // Beyond that, what the scan saves has to pay for the further launches and for
+  // the tail (its first threshold, pilot and top-k cost more the larger k is):
+  // the batch's codes, counted in 128-bit units, for k + 128 times 36000, and
+  // four times that for inner products, where the per-query scan prunes better.
+  // Of the 500 points with 1000 queries and more, this rule leaves 12 with over
+  // 3% and at most 10% against the per-query scan (four pairs alone: 80, up to
+  // 59%: 1000 queries x 4 probes, 100k x 96, k = 100: 0.174 ms per query, 0.262
+  // so). Below a thousand queries the tail's last wave is mostly idle.
+  const double pairs = (double)nq * a.mean_probes;
+  if (nq < 1000 || pairs < 4.0 * a.X->K) return false;
+  const double work = pairs * a.X->n / a.X->K * a.X->dpad / 128.0;
+  return work >= 36000.0 * (a.k + 128) * (a.X->metric != RABITQ_METRIC_L2 ? 4.0 : 1.0);
+}
+
+void expect_probes(SearchArgs& a) {
+  const float most = (float)std::min(a.nprobe, a.X->K);
+  a.mean_probes = a.pred ? std::min(most, a.pred->mean_nprobe()) : most;
 }
 
 size_t bucket_bytes(const SearchArgs& a, int64_t nq) {

@@ -672,6 +672,8 @@ int predictor_train_dev(const rabitq_index* X, const float* Q, int64_t nt, const
   pr->mult = h_mult[pick];
   pr->val_recall = (float)(h_cov[pick] / total);
   pr->val_mean_nprobe = (float)((double)h_np[pick] / (double)nval);
+  pr->mean_at.resize(kGrid);
+  for (int i = 0; i < kGrid; ++i) pr->mean_at[i] = (float)((double)h_np[i] / (double)nval);
   pr->train_loss = (float)(h_acc[0] / (double)ntr);
   pr->val_loss = (float)(h_acc[1] / (double)nval);
   pr->n_train = ntr;

@@ -2714,6 +2714,7 @@ void resolve_tile(const rabitq_index* X, int k, int nprobe, int32_t* path, int32
 int search_dev(const SearchArgs& a_in, cudaStream_t s) {
   SearchArgs a = a_in;
   const bool auto_path = a.scan_path == RABITQ_SCAN_AUTO;
+  expect_probes(a);
   a.tile_layout = a.layout;
   resolve_tile(a.X, a.k, a.nprobe, &a.scan_path, &a.tile_layout, &a.ppl, &a.stage);
   if (a.scan_path == RABITQ_SCAN_TC) {

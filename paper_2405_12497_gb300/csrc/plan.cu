@@ -161,6 +161,7 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
   a.scan_path = RABITQ_SCAN_POPC;  // plans run the popcount scan
   a.stage_ms = nullptr;
   a.pred = pr;
+  expect_probes(a);
   P->nq_max = nq_max;
   int grid = 0;
   int st = fused_grid(a, &grid);

@@ -159,3 +159,32 @@ def test_few_long_lists_do_not_hold_up_a_batch(R):
     assert torch.equal(ids, ids_r)
     assert torch.equal(dist.view(torch.int32), dist_r.view(torch.int32))
     assert t < 0.9 * t_ref
+
+
+# batches whose scan is too short to pay for the bucket-major launches: AUTO is
+# no slower than the per-query scan (1.3 to 1.6 times its time where it took the
+# other one)
+@pytest.mark.parametrize("metric,K,k,nprobe", [("l2", 256, 100, 4), ("l2", 256, 256, 8),
+                                               ("ip", 1024, 100, 16)])
+def test_short_scans_stay_per_query(R, metric, K, k, nprobe):
+    import torch
+    rng = np.random.default_rng(4)
+    data, Q = _mix(rng, 100_000, 96, comps=1000), _mix(rng, 1000, 96, comps=1000)
+    G = R.Index.build(data, K, seed=2, code_bits=128, kmeans_iters=3, metric=metric)
+
+    def best(**kw):
+        plan = R.Plan(G, k, nprobe, 1000, **kw)
+        plan.queries.copy_(torch.from_numpy(Q).cuda())
+        times = []
+        for _ in range(12):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            plan.run(1000)
+            e1.record()
+            e1.synchronize()
+            times.append(e0.elapsed_time(e1))
+        plan.sync()
+        return min(times[2:])
+
+    t, t_ref = best(), best(layout=R.LAYOUT_CTA, staging=R.STAGING_OFF)
+    assert t < 1.1 * t_ref
