@@ -411,9 +411,13 @@ int rabitq_autotune(rabitq_index* idx, const float* queries, int64_t nq, int32_t
  *                            applies: D' of 128 or 256, B_q = 4, k <= 128)
  *   {TC}                     bucket-major tensor-core products (an overflow
  *                            of its lists rules it out)
+ *   {POPC, AUTO}             the bucket-major scan that AUTO takes for large
+ *                            batches; only where it takes it for this one
  * Every candidate returns identical results. AUTO searches take the fastest
- * tile; plans, which run the popcount scan, take the fastest popcount tile.
- * best receives the chosen tile
+ * tile; plans, which do not run {TC}, take the fastest of the others. A large
+ * batch whose class was tuned with a batch too small for {POPC, AUTO} takes
+ * that scan as if it were not tuned; of a class where it was timed and was not
+ * the fastest no batch takes it. best receives the chosen tile
  * (time_ms its best time); all (may be NULL) receives up to cap candidates,
  * *n_all their count (time_ms -1 for one that could not run). reps >= 1
  * timed runs each after a warm-up run. Not thread-safe against searches on
@@ -421,7 +425,8 @@ int rabitq_autotune(rabitq_index* idx, const float* queries, int64_t nq, int32_t
  */
 typedef struct {
   int32_t scan_path;   /* RABITQ_SCAN_POPC or RABITQ_SCAN_TC             */
-  int32_t scan_layout; /* RABITQ_LAYOUT_CTA or _WARP (popcount path)      */
+  int32_t scan_layout; /* RABITQ_LAYOUT_CTA or _WARP (popcount path);
+                          _AUTO: bucket by bucket                         */
   int32_t lane_pairs;  /* codes per lane per step (warp layout), else 0   */
   int32_t staging;     /* RABITQ_STAGING_OFF or _BULK (CTA layout)        */
   float time_ms;       /* best measured time of one search of the sample  */
@@ -490,8 +495,9 @@ int rabitq_plan_search(rabitq_plan* plan, const float* queries, int64_t nq, int6
  * the number of entries written (0 without collect_stats). */
 int rabitq_plan_stats(rabitq_plan* plan, float* ms, int32_t cap);
 
-/* The tile a plan runs (its AUTO options resolved when the plan was made:
- * the index's tuned tile for its shape, else the defaults); time_ms is 0. */
+/* The tile a plan runs for a batch of nq_max (its AUTO options resolved when
+ * the plan was made: the index's tuned tile for its shape, else the defaults);
+ * time_ms is 0. */
 int rabitq_plan_tile(const rabitq_plan* plan, rabitq_tile* out);
 
 /* Release a plan (NULL is a no-op). */

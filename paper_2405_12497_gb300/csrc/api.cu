@@ -447,6 +447,24 @@ int rabitq_search_learned(const rabitq_index* idx, const rabitq_predictor* pr,
                        nullptr, pr);
 }
 
+// Whether a search with these options scans bucket by bucket.
+static bool runs_by_bucket(const rabitq_index* X, int64_t nq, int32_t k, int32_t nprobe,
+                           int32_t bq, const rabitq_search_opts& o) {
+  SearchArgs a{};
+  a.X = X;
+  a.nq = nq;
+  a.k = k;
+  a.nprobe = nprobe;
+  a.bq = bq;
+  a.cand_cap = o.max_candidates ? o.max_candidates : 65536;
+  a.scan_path = RABITQ_SCAN_POPC;
+  a.layout = o.scan_layout;
+  a.ppl = o.lane_pairs;
+  a.stage = o.scan_staging;
+  resolve_search(a);
+  return bucket_applies(a, query_chunk(X, nq));
+}
+
 int rabitq_autotune(rabitq_index* X, const float* queries, int64_t nq, int32_t k,
                     int32_t nprobe, int32_t bq, float eps0, int32_t reps,
                     const rabitq_search_opts* opts_in, int32_t* chosen, float* times_ms) {
@@ -508,6 +526,7 @@ int rabitq_autotune(rabitq_index* X, const float* queries, int64_t nq, int32_t k
   if (st_all != RABITQ_OK) return st_all;
   const int pick = (best[1] >= 0.0f && best[1] < best[0]) ? RABITQ_SCAN_TC : RABITQ_SCAN_POPC;
   X->tuned_path = pick;
+  X->tuned_bucket = runs_by_bucket(X, nq, k, nprobe, bq, opts);
   if (chosen) *chosen = pick;
   if (times_ms) {
     times_ms[0] = best[0];
@@ -554,7 +573,7 @@ int rabitq_autotune_tiles(rabitq_index* X, const float* queries, int64_t nq, int
   // the candidates: the warp layout only where it applies
   const bool warp_ok = bq == 4 && k <= 128 && X->d <= 256 && (X->W == 2 || X->W == 4);
   const bool stage_ok = bq == 4 && (X->W == 2 || X->W == 4);
-  rabitq_tile cand[6];
+  rabitq_tile cand[7];
   int nc = 0;
   cand[nc++] = rabitq_tile{RABITQ_SCAN_POPC, RABITQ_LAYOUT_CTA, 0, RABITQ_STAGING_OFF, -1.0f};
   if (stage_ok)
@@ -564,6 +583,22 @@ int rabitq_autotune_tiles(rabitq_index* X, const float* queries, int64_t nq, int
     cand[nc++] = rabitq_tile{RABITQ_SCAN_POPC, RABITQ_LAYOUT_WARP, 2, RABITQ_STAGING_OFF, -1.0f};
   }
   cand[nc++] = rabitq_tile{RABITQ_SCAN_TC, 0, 0, 0, -1.0f};
+  // the bucket-major scan, if AUTO takes it for this batch (an earlier verdict
+  // on the class aside, which stays should the tuning fail)
+  rabitq_index::Tile& t = X->tune[tile_class_k(k)][tile_class_np(std::min(nprobe, X->K))];
+  struct Keep {
+    rabitq_index::Tile& slot;
+    rabitq_index::Tile old;
+    bool done = false;
+    ~Keep() {
+      if (!done) slot = old;
+    }
+  } keep{t, t};
+  t = rabitq_index::Tile{};
+  opts.scan_layout = opts.lane_pairs = opts.scan_staging = 0;
+  const int by_bucket = runs_by_bucket(X, nq, k, nprobe, bq, opts) ? nc : -1;
+  if (by_bucket >= 0)
+    cand[nc++] = rabitq_tile{RABITQ_SCAN_POPC, RABITQ_LAYOUT_AUTO, 0, RABITQ_STAGING_AUTO, -1.0f};
   EventSet<2> ev;
   RBQ_CHECK(ev.create());
   // time with the warp-layout batch rule waived (the tuned tile is then
@@ -596,11 +631,13 @@ int rabitq_autotune_tiles(rabitq_index* X, const float* queries, int64_t nq, int
   for (int c = 1; c < nc; ++c) {
     if (cand[c].time_ms < 0.0f) continue;
     if (cand[c].time_ms < cand[pick].time_ms) pick = c;
-    if (cand[c].scan_path == RABITQ_SCAN_POPC && cand[c].time_ms < cand[pick_popc].time_ms)
+    if (cand[c].scan_path == RABITQ_SCAN_POPC && c != by_bucket &&
+        cand[c].time_ms < cand[pick_popc].time_ms)
       pick_popc = c;
   }
-  rabitq_index::Tile& t = X->tune[tile_class_k(k)][tile_class_np(std::min(nprobe, X->K))];
+  keep.done = true;
   t.valid = 1;
+  t.bucket = by_bucket < 0 ? 0 : (cand[by_bucket].time_ms <= cand[pick_popc].time_ms ? 1 : 2);
   t.path = cand[pick].scan_path;
   t.layout = cand[pick_popc].scan_layout;
   t.ppl = cand[pick_popc].lane_pairs;

@@ -34,11 +34,13 @@ struct rabitq_index {
   int32_t kp = 0;
   int32_t tuned_path = 0;         // scan path AUTO uses (rabitq_autotune)
   int32_t tuned_layout = 0;       // scan layout AUTO uses (rabitq_autotune), 0 = default
+  int32_t tuned_bucket = 0;       // tuned_path was timed against the bucket-major scan
   // tiles chosen by rabitq_autotune_tiles per (k class, nprobe class)
-  // (path: the fastest overall; layout, ppl: the fastest popcount tile,
-  // which plans run)
+  // (path: the fastest overall; layout, ppl: the fastest per-query popcount
+  // tile; bucket: the bucket-major scan was not timed (0), or was the faster
+  // (1) or the slower (2) of it and that tile)
   struct Tile {
-    int32_t valid, path, layout, ppl, stage;
+    int32_t valid, path, layout, ppl, stage, bucket;
   } tune[4][4] = {};
   void* ptb = nullptr;            // dpad x kp BF16
   float* ptf = nullptr;           // dpad x kp TF32-rounded FP32
@@ -285,6 +287,10 @@ struct SearchArgs {
   // probes per query that are expected: nprobe, or the predictor's mean at the
   // multiplier it had when the call or plan was made (expect_probes)
   float mean_probes = 0.0f;
+  // the tuner's verdict on the bucket-major scan (rabitq_index::Tile::bucket),
+  // and whether bulk-copy staging was asked for (not tuned): resolve_search
+  int32_t bucket_tuned = 0;
+  int32_t bulk_asked = 0;
   // bulk-copy staging of the CTA layout's scan rounds (RABITQ_STAGING_*;
   // AUTO resolves to the tuned or default choice)
   int32_t stage = 0;
@@ -293,6 +299,12 @@ struct SearchArgs {
 // from the index's tuned tiles for the shape's class, else the defaults.
 void resolve_tile(const rabitq_index* X, int k, int nprobe, int32_t* path, int32_t* layout,
                   int32_t* ppl, int32_t* stage);
+// The same for a search's arguments, with everything bucket_applies reads; a
+// tensor-core path that was tuned without the bucket-major scan among its
+// rivals gives way to it.
+void resolve_search(SearchArgs& a);
+// queries scanned together by a search of a.nq (its centroid scores' chunk)
+int64_t query_chunk(const rabitq_index* X, int64_t nq);
 int tile_class_k(int k);
 int tile_class_np(int nprobe);
 int search_dev(const SearchArgs& a, cudaStream_t s);

@@ -1502,7 +1502,7 @@ int pack_rows(rabitq_index* X, cudaStream_t s) {
 
 bool bucket_applies(const SearchArgs& a, int64_t nq) {
   if (!a.allow_bucket || a.trace || a.bq > 4 || a.k > 256 || a.cand_cap < 65536) return false;
-  if (a.layout != RABITQ_LAYOUT_AUTO || a.stage == RABITQ_STAGING_BULK) return false;
+  if (a.layout != RABITQ_LAYOUT_AUTO || a.bulk_asked || a.bucket_tuned == 2) return false;
   // Measured against the per-query scan on eight indexes (100k x 96 to 2M x 256,
   // D' 128 to 1024, L2 and inner products), k 1 to 256, 320 to 10k queries, 4 to
   // 128 probes. Below about four pairs per bucket the tiles are mostly padding.

@@ -2711,12 +2711,28 @@ void resolve_tile(const rabitq_index* X, int k, int nprobe, int32_t* path, int32
     *stage = t.valid && t.stage ? t.stage : RABITQ_STAGING_OFF;
 }
 
-int search_dev(const SearchArgs& a_in, cudaStream_t s) {
-  SearchArgs a = a_in;
+int64_t query_chunk(const rabitq_index* X, int64_t nq) {
+  return std::max<int64_t>(1, std::min<int64_t>(nq, (int64_t(1) << 28) / X->K));
+}
+
+void resolve_search(SearchArgs& a) {
+  const rabitq_index* X = a.X;
+  const rabitq_index::Tile& t = X->tune[tile_class_k(a.k)][tile_class_np(a.nprobe)];
   const bool auto_path = a.scan_path == RABITQ_SCAN_AUTO;
   expect_probes(a);
   a.tile_layout = a.layout;
-  resolve_tile(a.X, a.k, a.nprobe, &a.scan_path, &a.tile_layout, &a.ppl, &a.stage);
+  a.bulk_asked = a.stage == RABITQ_STAGING_BULK;
+  a.bucket_tuned = t.valid ? t.bucket : 0;
+  resolve_tile(X, a.k, a.nprobe, &a.scan_path, &a.tile_layout, &a.ppl, &a.stage);
+  if (auto_path && a.scan_path == RABITQ_SCAN_TC && !(t.valid ? t.bucket : X->tuned_bucket) &&
+      bucket_applies(a, query_chunk(X, a.nq)))
+    a.scan_path = RABITQ_SCAN_POPC;
+}
+
+int search_dev(const SearchArgs& a_in, cudaStream_t s) {
+  SearchArgs a = a_in;
+  const bool auto_path = a.scan_path == RABITQ_SCAN_AUTO;
+  resolve_search(a);
   if (a.scan_path == RABITQ_SCAN_TC) {
     const int st = search_dev_tc(a, s);
     if (!(auto_path && st == RABITQ_EOVERFLOW)) return st;
@@ -2745,7 +2761,7 @@ int search_popc_run(const SearchArgs& a, bool* by_bucket_out, cudaStream_t s) {
   const int per_sm = fs.per_sm;
 
   // query chunks bound the centroid-distance scratch (<= 256 Mi floats)
-  const int64_t qchunk = std::max<int64_t>(1, std::min<int64_t>(a.nq, (int64_t(1) << 28) / K));
+  const int64_t qchunk = query_chunk(X, a.nq);
   const int64_t full = (int64_t)sms * per_sm;
   const int64_t grid = std::min<int64_t>(qchunk, full);
   // a batch too small to fill the GPU splits each query's probes over CTAs

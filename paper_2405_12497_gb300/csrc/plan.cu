@@ -155,13 +155,11 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
   a.layout = opts.scan_layout;
   a.ppl = opts.lane_pairs;
   a.stage = opts.scan_staging;
-  // the plan keeps the tile resolved now (later tuning does not change it)
-  a.tile_layout = a.layout;
-  resolve_tile(X, k, nprobe, &a.scan_path, &a.tile_layout, &a.ppl, &a.stage);
-  a.scan_path = RABITQ_SCAN_POPC;  // plans run the popcount scan
   a.stage_ms = nullptr;
   a.pred = pr;
-  expect_probes(a);
+  // the plan keeps the tile resolved now (later tuning does not change it)
+  resolve_search(a);
+  a.scan_path = RABITQ_SCAN_POPC;  // plans run the popcount scan
   P->nq_max = nq_max;
   int grid = 0;
   int st = fused_grid(a, &grid);
@@ -271,7 +269,13 @@ int rabitq_plan_search(rabitq_plan* P, const float* queries, int64_t nq, int64_t
 int rabitq_plan_tile(const rabitq_plan* P, rabitq_tile* out) {
   if (!P || !out) return fail(RABITQ_EINVAL, "rabitq_plan_tile: null argument");
   out->scan_path = RABITQ_SCAN_POPC;
+  out->time_ms = 0.0f;
   const rabitq_index* X = P->a.X;
+  if (bucket_applies(P->a, P->nq_max)) {  // (batches of nq_max)
+    out->scan_layout = RABITQ_LAYOUT_AUTO;
+    out->lane_pairs = out->staging = 0;
+    return RABITQ_OK;
+  }
   const bool warp = P->a.tile_layout == RABITQ_LAYOUT_WARP && P->a.bq == 4 && P->a.k <= 128 &&
                     X->d <= 256 && (X->W == 2 || X->W == 4);
   out->scan_layout = warp ? RABITQ_LAYOUT_WARP : RABITQ_LAYOUT_CTA;
@@ -280,7 +284,6 @@ int rabitq_plan_tile(const rabitq_plan* P, rabitq_tile* out) {
                          (X->W == 2 || X->W == 4)
                      ? RABITQ_STAGING_BULK
                      : RABITQ_STAGING_OFF;
-  out->time_ms = 0.0f;
   return RABITQ_OK;
 }
 

@@ -75,9 +75,11 @@ class Tile(C.Structure):
                 ("lane_pairs", C.c_int32), ("staging", C.c_int32), ("time_ms", C.c_float)]
 
     def as_dict(self):
+        layout = {1: "cta-per-query", 2: "warp-per-query"}.get(self.scan_layout, self.scan_layout)
+        if self.scan_path == SCAN_POPC and self.scan_layout == LAYOUT_AUTO:
+            layout = "bucket-major"  # AUTO's scan of large batches
         return {"scan_path": {1: "popcount", 2: "tensor-core"}.get(self.scan_path, self.scan_path),
-                "layout": {1: "cta-per-query", 2: "warp-per-query"}.get(self.scan_layout,
-                                                                        self.scan_layout),
+                "layout": layout,
                 "lane_pairs": self.lane_pairs,
                 "staging": {1: "off", 2: "bulk-copy"}.get(self.staging, self.staging),
                 "time_ms": round(float(self.time_ms), 4)}

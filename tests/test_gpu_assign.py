@@ -72,3 +72,24 @@ def test_device_rows_at_any_address(R, oracle_mod):
     cent, assign, _ = oracle_mod.kmeans(data, 80, 2, 5, threads=4)
     assert np.array_equal(G.centroids().view(np.uint32), cent.view(np.uint32))
     assert np.array_equal(G.assign(), assign)
+
+
+def test_row_chunks(R):
+    """More rows than a GiB of operand tiles holds (8388608 at up to 64
+    dimensions): the rows at the chunks' ends are assigned as in builds of
+    their own, small enough for the canonical scan."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    chunk, d, K = 1 << 23, 16, 70
+    cen = torch.randn((K, d), generator=g, device="cuda")
+    n = chunk + 5001
+    data = cen[torch.randint(0, K, (n,), generator=g, device="cuda")]
+    data += 0.5 * torch.randn((n, d), generator=g, device="cuda")
+    G = R.Index.build(data, K, seed=2, centroids=cen)
+    got = G.assign()
+    for at in (0, chunk - 4000, chunk, n - 4000):
+        S = R.Index.build(data[at:at + 4000].contiguous(), K, seed=2, centroids=cen)
+        assert np.array_equal(got[at:at + 4000], S.assign()), at
+        S.free()
+    G.free()
