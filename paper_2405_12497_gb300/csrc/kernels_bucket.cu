@@ -8,7 +8,9 @@
 // estimator, its bound and the candidates come from the accumulator:
 //
 //   1. bucket_tau0_kernel   per query, the k-th smallest upper bound of its
-//                           first codes (nearest probes): tau0 >= tau_ub
+//                           first codes (nearest probes): tau0 >= tau_ub. Of a
+//                           short query these are all its codes: its
+//                           candidates, and steps 2 to 4 are without it
 //   2. bucket_count / bucket_plan / bucket_quant: (query, probe) pairs
 //                           grouped by bucket, quantized (§3.3.1) into
 //                           operand rows; work items {bucket, pairs, codes};
@@ -63,6 +65,7 @@ constexpr int kGMmaWarp = kGEpiWarps + kGProdWarps, kGItemWarp = kGMmaWarp + 1;
 constexpr int kGThreads = (kGItemWarp + 1) * 32;
 constexpr int kGTilesPerItem = 4;        // code tiles per work item
 constexpr int kGPad = 16;                // a bucket's pair slots start at a multiple of this
+constexpr int kQJ = 4;                   // probes per quantization run
 constexpr int kGTau0Probes = 16;         // probes the first threshold may look at
 constexpr float kGSlack = 0x1.0p-18f;    // prefilter slack (bucket_scan_kernel)
 constexpr int kGLevels = 6;              // list capacities: the even share << level
@@ -146,34 +149,62 @@ __device__ __forceinline__ int probes_of(const FusedParams& P, int64_t q) {
   return P.nprobe_q ? min(max(P.nprobe_q[q], 1), P.nprobe) : P.nprobe;
 }
 
-// One warp per query (learned counts are mostly far below nprobe). Also the
-// entries that all candidate lists would take at each level of capacity
+// Whether the first threshold looks at all codes of a query (np probes).
+__device__ __forceinline__ bool short_query(int codes, int np, int want_max) {
+  return codes <= want_max && np <= kGTau0Probes;
+}
+
+// One warp per query (learned counts are mostly far below nprobe); short ones
+// are marked and not counted. Of the others also, where counts differ, the runs
+// of kQJ probes for the quantization, and of all the entries that all candidate lists would take at each level of capacity
 // (share << level, and never more than the query's codes): lsum.
-__global__ void __launch_bounds__(256) bucket_count_kernel(FusedParams P, int share,
+__global__ void __launch_bounds__(256) bucket_count_kernel(FusedParams P, int share, int want_max,
                                                            int32_t* __restrict__ bcnt,
-                                                           unsigned long long* __restrict__ lsum) {
-  __shared__ int s_codes[8];
+                                                           unsigned long long* __restrict__ lsum,
+                                                           int* __restrict__ is_short,
+                                                           int* __restrict__ nruns,
+                                                           int2* __restrict__ runs) {
+  __shared__ int s_codes[8], s_runs[8], s_base;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int codes = 0;
+  int codes = 0, nr = 0;
   if (q < P.nq) {
     const int np = probes_of(P, q);
+    int first = -1;  // the lane's only probe of a query that may be short
     for (int j = lane; j < np; j += 32) {
       const int c = P.probe_ids[q * P.nprobe + j];
       if (c >= 0) {
-        atomicAdd(bcnt + c, 1);
+        if (np > kGTau0Probes) atomicAdd(bcnt + c, 1); else first = c;
         codes += __ldg(P.bucket_off + c + 1) - __ldg(P.bucket_off + c);
       }
     }
+    __syncwarp();
+    codes = __reduce_add_sync(kFull, codes);
+    const bool brief = short_query(codes, np, want_max);
+    if (first >= 0 && !brief) atomicAdd(bcnt + first, 1);
+    if (lane == 0) is_short[q] = brief;
+    if (P.nprobe_q && !brief) nr = (np + kQJ - 1) / kQJ;
   }
-  codes = __reduce_add_sync(kFull, codes);
-  if (lane == 0) s_codes[wid] = codes;
+  if (lane == 0) {
+    s_codes[wid] = codes;
+    s_runs[wid] = nr;
+  }
   __syncthreads();
+  if (P.nprobe_q && threadIdx.x == 32) {
+    int sum = 0;
+    for (int w = 0; w < 8; ++w) sum += s_runs[w];
+    s_base = atomicAdd(nruns, sum);
+  }
   if (threadIdx.x < kGLevels) {
     unsigned long long sum = 0;
     for (int w = 0; w < 8; ++w) sum += min((int64_t)s_codes[w], (int64_t)share << threadIdx.x);
     atomicAdd(lsum + threadIdx.x, sum);
   }
+  if (!P.nprobe_q) return;
+  __syncthreads();
+  int at = s_base;
+  for (int w = 0; w < wid; ++w) at += s_runs[w];
+  for (int i = lane; i < nr; i += 32) runs[at + i] = make_int2((int)q, i * kQJ);
 }
 
 // Exclusive block scan of one int per thread (1024 threads); returns the
@@ -258,33 +289,48 @@ __global__ void __launch_bounds__(1024) bucket_plan_kernel(const int32_t* __rest
 // taken from a multiplication by 1 / Delta unless the sum falls within 3e-5
 // of an integer (the multiplied form is within 5e-6 of the correctly rounded
 // one for x < 16), where the division decides.
-constexpr int kQJ = 4;
-// Warps per query (each takes every quant_runs-th run): learned counts are
-// mostly far below nprobe, and a warp per possible run was mostly warps
-// without work (nprobe_max 256, 7.6 probes on average: 92 us per 8000 queries).
+// With one count for all queries a warp takes every quant_runs-th run of its
+// query. LISTED: the warps take the runs in turn, from a list
+// (bucket_count_kernel): per-query counts are mostly far below nprobe, and a
+// warp per possible run was mostly warps without work (nprobe_max 256, 7.6
+// probes on average: 92 us per 8000 queries), while with four warps to each
+// query most idled as those of 100 probes and more held up the rest (52 us; so
+// 29; with one count the list is 1 to 2% of a search slower).
 __host__ __device__ inline int quant_runs(int nprobe) {
   const int r = (nprobe + kQJ - 1) / kQJ;
   return r < 4 ? r : 4;
 }
+template <bool LISTED>
 __global__ void __launch_bounds__(256) bucket_quant_kernel(FusedParams P,
+                                                           const int* __restrict__ is_short,
+                                                           const int* __restrict__ nruns,
+                                                           const int2* __restrict__ list,
                                                            const int32_t* __restrict__ boff,
                                                            int32_t* __restrict__ bfill,
                                                            uint8_t* __restrict__ qop,
                                                            float4* __restrict__ smeta,
                                                            float* __restrict__ spsum,
                                                            int32_t* __restrict__ sq) {
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
+  const int w = (blockIdx.x * 256 + threadIdx.x) >> 5;
   const int runs = quant_runs(P.nprobe);
-  const int64_t q = w / runs;
-  if (q >= P.nq) return;
-  const int np = probes_of(P, q);
+  int64_t q = w / runs;
+  if (!LISTED && (q >= P.nq || is_short[q])) return;
+  // items: runs of the list, or first probes of the query's runs
+  const int end = LISTED ? *nruns : probes_of(P, q);
+  const int step = LISTED ? (int)gridDim.x * 8 : runs * kQJ;
   const int dpad = P.dpad;
   const int qmax = (1 << P.bq) - 1;
-  const float* rq = P.rq + q * dpad;
   const uint32_t sub = (uint32_t)(lane >> 1) & 3u;  // byte of the operand word
-  for (int j0 = (int)(w - q * runs) * kQJ; j0 < np; j0 += runs * kQJ) {
-  const int nj = min(kQJ, np - j0);
+  for (int i = LISTED ? w : (int)(w - q * runs) * kQJ; i < end; i += step) {
+  int j0 = i;
+  if (LISTED) {
+    const int2 run = __ldg(list + i);
+    q = run.x;
+    j0 = run.y;
+  }
+  const int nj = min(kQJ, (LISTED ? probes_of(P, q) : end) - j0);
+  const float* rq = P.rq + q * dpad;
   // lane j < nj: pair j's cluster, slot and constants
   int c_l = -1, slot_l = 0, sum_l = 0;
   float vl_l = 0.0f, delta_l = 0.0f, add_l = 0.0f, nq2_l = 0.0f;
@@ -388,8 +434,10 @@ struct ListPool {
 // tau0 of a query: the k-th smallest upper bound of its first `want` codes
 // (in probe order, at most kGTau0Probes probes), +inf when there are fewer
 // than k. The k-th smallest of any subset bounds tau_ub from above. Of a
-// query with at most want_max codes all are looked at: that is tau_ub itself,
-// and tau0 = -inf keeps pass 1 from the query. Also clears the query's hit
+// short query (at most want_max codes in kGTau0Probes probes) all are looked
+// at: that is tau_ub itself, the candidates are written here, and tau0 = -inf
+// keeps the tau kernel from the query: its pairs are not grouped, quantized or
+// scanned. Also clears the query's hit
 // counters and takes its candidate list from the pool, at the highest level at
 // which all lists fit (level 0 does: the pool has a share for each). One CTA
 // per query.
@@ -398,7 +446,8 @@ struct ListPool {
 template <int WT, int BQT>
 __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
     FusedParams P, int want_max, ListPool lp, float* __restrict__ tau0, float* __restrict__ taub,
-    int* __restrict__ ucnt, int* __restrict__ lcnt, int2* __restrict__ lrow) {
+    int* __restrict__ ucnt, int* __restrict__ lcnt, int2* __restrict__ lrow,
+    int4* __restrict__ list) {
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ SelState s_sel;
   __shared__ float4 s_meta[kGTau0Probes];
@@ -416,6 +465,7 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
   uint32_t* ub = reinterpret_cast<uint32_t*>(smem + sizeof(uint64_t) * kGTau0Probes * bq * W);
   int* hist = reinterpret_cast<int*>(ub + want_max);
   uint32_t* coll = reinterpret_cast<uint32_t*>(hist + kHistBins);
+  float2* both = reinterpret_cast<float2*>(coll + 256);  // a short query's LB, estimate
   const int np_all = probes_of(P, q), np = min(np_all, kGTau0Probes);
   // the codes to look at: a third of the query's codes where that is fewer
   // than want_max (at least 4 k): a code costs here over twice what it costs
@@ -430,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
   __syncthreads();
   codes = 0;
   for (int w = 0; w < kThreads / 32; ++w) codes += s_sel.warp_cnt[w];
-  const bool all = codes <= want_max && np_all <= kGTau0Probes;  // tau0 is tau_ub then
+  const bool all = short_query(codes, np_all, want_max);  // tau0 is tau_ub then
   const int want = all ? codes : min(want_max, max(codes / 3, 4 * P.k));
   if (wid == 0) {  // the probes that hold the first `want` codes
     int len = 0;
@@ -450,13 +500,15 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
   if (tid == 0) {
     ucnt[q] = 0;
     lcnt[q] = 0;
-    int l = kGLevels - 1;
-    while (l > 0 && lp.sum[l] > lp.size) --l;
-    const int cap = (int)min((int64_t)codes, (int64_t)lp.share << l);
-    lrow[q] = make_int2((int)atomicAdd(lp.used, (unsigned)cap), cap);
   }
   __syncthreads();
   const int m = s_np;
+  if (wid == kThreads / 32 - 1) {  // (a warp that seldom has a probe to quantize)
+    const bool fits = lane < kGLevels && lp.sum[lane] <= lp.size;
+    const int l = 31 - __clz((int)(__ballot_sync(kFull, fits) | 1u));
+    const int cap = (int)min((int64_t)codes, (int64_t)lp.share << l);
+    if (lane == 0) lrow[q] = make_int2((int)atomicAdd(lp.used, (unsigned)cap), cap);
+  }
   for (int j = wid; j < m; j += kThreads / 32) {
     const int64_t pj = q * P.nprobe + j;
     const float add = P.probe_dist[pj];
@@ -486,7 +538,9 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
     const float t1 = (float)(2 * ip - s_psum[j]);
     const float xq = __fadd_rn(__fmul_rn(mt.x, t1), __fmul_rn(mt.y, f.w));
     const float dist = __fsub_rn(__fadd_rn(f.x, mt.w), __fmul_rn(f.y, xq));
-    ub[t] = float_key(__fadd_rn(dist, __fmul_rn(f.z, mt.z)));
+    const float er = __fmul_rn(f.z, mt.z);
+    ub[t] = float_key(__fadd_rn(dist, er));
+    if (all) both[t] = make_float2(__fsub_rn(dist, er), dist);
   }
   __syncthreads();
   float tau = __int_as_float(0x7f800000);
@@ -499,6 +553,25 @@ __global__ void __launch_bounds__(kThreads, WT == 2 ? 6 : 4) bucket_tau0_kernel(
     tau0[q] = all ? __int_as_float(0xff800000) : tau;
     if (all) taub[q] = tau;
   }
+  if (!all) return;
+  int4* L = list + lrow[q].x;  // (n entries at most: the query's codes)
+  if (tid == 0) s_np = 0;
+  __syncthreads();
+  j = 0;
+  for (int t0 = 0; t0 < n; t0 += kThreads) {
+    const int t = t0 + tid;
+    float2 e = make_float2(0.0f, 0.0f);
+    if (t < n) e = both[t];
+    const bool in = t < n && e.x <= tau;
+    const int slot = warp_reserve(in, &s_np);
+    if (in) {
+      while (s_pref[j + 1] <= t) ++j;
+      L[slot] = make_int4(s_pbeg[j] + (t - s_pref[j]), __float_as_int(e.x), __float_as_int(e.y),
+                          __float_as_int(key_float(ub[t])));
+    }
+  }
+  __syncthreads();
+  if (tid == 0) lcnt[q] = s_np;
 }
 
 // tau_ub of a query: the k-th smallest upper bound of its pass-1 list (which
@@ -651,15 +724,6 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
         tau[u] = in ? __ldg(P.tau + q[u]) : __int_as_float(0xff800000);
         if (MODE == 2) lr[u] = in ? __ldg(P.lrow + q[u]) : make_int2(0, 0);
       }
-      if (MODE == 1 && x.c >= 0) {  // an item whose queries all know their tau_ub
-        float best = tau[0];
-#pragma unroll
-        for (int u = 1; u < kGN / 32; ++u) best = fmaxf(best, tau[u]);
-        if (!__any_sync(kFull, best != __int_as_float(0xff800000))) {
-          --it;
-          continue;
-        }
-      }
       if (it >= 2) ok = __all_sync(kFull, pd_wait(smem_u32(&s_mempty[buf]), ((it >> 1) - 1) & 1u, &s_fail));
       if (!ok) {
         s_fail = 1;
@@ -671,7 +735,7 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
       for (int u = 0; u < kGN / 32; ++u) {
         const int j = u * 32 + lane;
         if (j >= padded) continue;
-        const bool none = j >= x.cols || tau[u] == __int_as_float(0xff800000);
+        const bool none = j >= x.cols;
         const float thr = none ? __int_as_float(0xff800000)
                                : (tau[u] - m[u].w) + kGSlack * (fabsf(m[u].w) + fabsf(tau[u]));
         M.ex[j] = m[u];
@@ -1296,7 +1360,7 @@ __global__ void __launch_bounds__(kThreads, 4) bucket_tail_kernel(TailParams T) 
     // are ranked against each other; the dropped ones do no harm in the list
     // (the end ranks again).
     unsigned long long T1 = ~0ull;
-    if (pilot >= k) {
+    if (pilot >= k && !pilot_all) {  // (without other candidates T1 is of no use)
       const int nt = s_top;
       if (nt <= kThreads) {
         const unsigned long long mine = tid < nt ? topk[tid] : ~0ull;
@@ -1393,7 +1457,7 @@ size_t tail_smem_bytes(int ct, int ce, int sk, int d) {
          align_up(sizeof(float) * d, 16) + 32 * (size_t)((d + 15) / 16);
 }
 
-typedef void (*Tau0Fn)(FusedParams, int, ListPool, float*, float*, int*, int*, int2*);
+typedef void (*Tau0Fn)(FusedParams, int, ListPool, float*, float*, int*, int*, int2*, int4*);
 Tau0Fn pick_tau0(int W, int bq) {
   if (bq == 4) {
     if (W == 2) return bucket_tau0_kernel<2, 4>;
@@ -1421,7 +1485,7 @@ struct BucketScratch {
   int32_t *bcnt, *bfill, *boff;
   int4* items;
   // [0] items, [16] the levels' sums (64-bit), [32] [64] work counters of the
-  // passes, [96] tail counter, [112] pool entries taken
+  // passes, [96] tail counter, [120] pool entries taken, [124] runs
   int* ctl;
   uint8_t* qop;
   float4* smeta;
@@ -1432,6 +1496,7 @@ struct BucketScratch {
   int2* lrow;
   uint32_t* ulist;
   int4* list;
+  int2* runs;  // {query, first probe}
   int* redo;  // [0] count, [32] the redo launch's work counter, list from [64]
   uint8_t* qrec;
   size_t bytes;
@@ -1467,6 +1532,9 @@ BucketScratch bucket_carve(const SearchArgs& a, int64_t nq, unsigned char* base)
   b.ucnt = reinterpret_cast<int*>(take(sizeof(int) * nq));
   b.lcnt = reinterpret_cast<int*>(take(sizeof(int) * nq));
   b.lrow = reinterpret_cast<int2*>(take(sizeof(int2) * nq));
+  const bool counts = a.pred || a.per_query_nprobe;
+  b.runs = reinterpret_cast<int2*>(
+      take(counts ? sizeof(int2) * nq * ((std::min(a.nprobe, X->K) + kQJ - 1) / kQJ) : 0));
   b.ulist = reinterpret_cast<uint32_t*>(take(sizeof(uint32_t) * nq * cap_upper(a.k)));
   b.list = reinterpret_cast<int4*>(take(sizeof(int4) * nq * list_share(a)));
   b.qrec = take((size_t)nq * query_stride(X->d));
@@ -1545,7 +1613,7 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
   RBQ_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   const Tau0Fn t0 = pick_tau0(X->W, a.bq);
   const size_t t0_smem = sizeof(uint64_t) * kGTau0Probes * a.bq * X->W + sizeof(uint32_t) * want +
-                         sizeof(int) * kHistBins + sizeof(uint32_t) * 256;
+                         sizeof(int) * kHistBins + sizeof(uint32_t) * 256 + sizeof(float2) * want;
   RBQ_CUDA(cudaFuncSetAttribute(t0, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
   const size_t scan_smem = bucket_smem_bytes(nt, X->dpad);
   RBQ_CUDA(cudaFuncSetAttribute(bucket_scan_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1582,15 +1650,21 @@ int bucket_search(const SearchArgs& a, const FusedParams& P0, unsigned char* scr
     RBQ_CUDA(cudaMemsetAsync(b.bcnt, 0, sizeof(int32_t) * (2 * K + 192), s));  // counts, ctl, redo
     ListPool lp;
     lp.sum = reinterpret_cast<unsigned long long*>(b.ctl + 16);
-    lp.used = reinterpret_cast<unsigned*>(b.ctl + 112);
+    lp.used = reinterpret_cast<unsigned*>(b.ctl + 120);
     lp.size = (unsigned)(per * share);
     lp.share = share;
     bucket_count_kernel<<<blocks(P.nq * 32, 256), 256, 0, s>>>(
-        P, share, b.bcnt, reinterpret_cast<unsigned long long*>(b.ctl + 16));
+        P, share, want, b.bcnt, reinterpret_cast<unsigned long long*>(b.ctl + 16), b.lcnt,
+        b.ctl + 124, b.runs);
     bucket_plan_kernel<<<1, 1024, 0, s>>>(b.bcnt, X->bucket_off, K, nt, b.boff, b.items, b.ctl);
-    bucket_quant_kernel<<<blocks(P.nq * quant_runs(P.nprobe) * 32, 256), 256, 0, s>>>(
-        P, b.boff, b.bfill, b.qop, b.smeta, b.spsum, b.sq);
-    t0<<<(unsigned)P.nq, kThreads, t0_smem, s>>>(P, want, lp, b.tau0, b.taub, b.ucnt, b.lcnt, b.lrow);
+    if (P.nprobe_q)
+      bucket_quant_kernel<true><<<(unsigned)(4 * sms), 256, 0, s>>>(
+          P, b.lcnt, b.ctl + 124, b.runs, b.boff, b.bfill, b.qop, b.smeta, b.spsum, b.sq);
+    else
+      bucket_quant_kernel<false><<<blocks(P.nq * quant_runs(P.nprobe) * 32, 256), 256, 0, s>>>(
+          P, b.lcnt, nullptr, nullptr, b.boff, b.bfill, b.qop, b.smeta, b.spsum, b.sq);
+    t0<<<(unsigned)P.nq, kThreads, t0_smem, s>>>(P, want, lp, b.tau0, b.taub, b.ucnt, b.lcnt, b.lrow,
+                                                  b.list);
     RBQ_CUDA(cudaGetLastError());
     BucketParams B;
     B.codes = X->codes;

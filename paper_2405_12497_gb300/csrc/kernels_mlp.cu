@@ -178,14 +178,20 @@ __global__ void __launch_bounds__(kInferThreads, 4) mlp_infer_kernel(
   const int64_t q0 = (int64_t)blockIdx.x * kQB;
   const int nqb = (int)(nq - q0 < kQB ? nq - q0 : kQB);
   w3[tid] = __bfloat162float(P[ow3 + tid]);
-  for (int i = tid; i < kQB * kF; i += blockDim.x) {
-    const int q = i / kF, j = i % kF;
-    float v = 0.0f;
-    if (q < nqb) {
-      v = feature(sel_dist + (q0 + q) * ld, navail, j, s0);
-      if (feat_out) feat_out[(q0 + q) * kF + j] = v;
+  constexpr int kEach = kQB * kF / kInferThreads;  // (their loads in flight together)
+  {
+    float v[kEach];
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const int i = u * kInferThreads + tid, q = i / kF;
+      v[u] = q < nqb ? feature(sel_dist + (q0 + q) * ld, navail, i % kF, s0) : 0.0f;
     }
-    xT[j * kQB + q] = v;
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const int i = u * kInferThreads + tid, q = i / kF, j = i % kF;
+      if (q < nqb && feat_out) feat_out[(q0 + q) * kF + j] = v[u];
+      xT[j * kQB + q] = v[u];
+    }
   }
   __syncthreads();
   // a warp: 32 unit groups of one half of the units, one query group
@@ -262,11 +268,24 @@ __global__ void __launch_bounds__(kInferThreads, 4) mlp_infer_kernel(
   }
   if (L.out_ids) {
     __syncthreads();
-    for (int i = tid; i < nqb * kF; i += blockDim.x) {
-      const int q = i / kF, j = i % kF;
-      if (j < s_np[q] && j < navail) {
-        L.out_ids[(q0 + q) * L.ldo + j] = L.sel_ids[(q0 + q) * ld + j];
-        L.out_dist[(q0 + q) * L.ldo + j] = sel_dist[(q0 + q) * ld + j];
+    int32_t id[kEach];
+    float ds[kEach];
+    bool in[kEach];
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const int i = u * kInferThreads + tid, q = i / kF, j = i % kF;
+      in[u] = q < nqb && j < s_np[q] && j < navail;
+      if (in[u]) {
+        id[u] = L.sel_ids[(q0 + q) * ld + j];
+        ds[u] = sel_dist[(q0 + q) * ld + j];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kEach; ++u) {
+      const int i = u * kInferThreads + tid, q = i / kF, j = i % kF;
+      if (in[u]) {
+        L.out_ids[(q0 + q) * L.ldo + j] = id[u];
+        L.out_dist[(q0 + q) * L.ldo + j] = ds[u];
       }
     }
   }

@@ -135,3 +135,25 @@ def test_plans_and_the_tuner_name_the_scan(R):
     ids, dist = G.search(Q, 10, 16)
     assert torch.equal(ids, want[0])
     assert torch.equal(dist.view(torch.int32), want[1].view(torch.int32))
+
+
+# a learned plan selects a large batch in two parts on two streams; queries of
+# few codes take their candidates from the first threshold, and a few probe
+# every bucket
+@pytest.mark.parametrize("nq,nprobe_max", [(4095, 48), (4099, 48), (6001, 200)])
+def test_learned_plans(R, nq, nprobe_max):
+    import torch
+    rng = np.random.default_rng(17)
+    data, Q = _mix(rng, 60_000, 128), torch.from_numpy(_mix(rng, nq, 128)).cuda()
+    G = R.Index.build(data, 200, seed=2, kmeans_iters=3)
+    pr = R.Predictor.train(G, torch.from_numpy(_mix(rng, 2048, 128)).cuda(), k=100,
+                           nprobe_max=nprobe_max, epochs=2, batch=512)
+    npq = G.predict_nprobe(pr, Q)
+    plan = R.Plan(G, 100, 0, nq, predictor=pr)
+    assert plan.tile()["layout"] == "bucket-major"
+    want = G.search(Q, 100, nprobe_max, per_query_nprobe=npq, layout=R.LAYOUT_CTA,
+                    staging=R.STAGING_OFF)
+    for ids, dist in (G.search_learned(pr, Q, 100), plan.search(Q), plan.search(Q)):
+        assert torch.equal(ids, want[0])
+        assert torch.equal(dist.view(torch.int32), want[1].view(torch.int32))
+    assert torch.equal(plan.nprobe[:nq], npq)
