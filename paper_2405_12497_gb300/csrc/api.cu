@@ -43,6 +43,7 @@ int dev_alloc(T** p, size_t count) {
   cudaError_t e = cudaMalloc((void**)p, sizeof(T) * count);
   if (e != cudaSuccess) {
     *p = nullptr;
+    cudaGetLastError();  // (the next launch's check must not find it)
     return fail(RABITQ_ENOMEM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
   }
   return RABITQ_OK;
@@ -257,8 +258,12 @@ int rabitq_build(const float* data, int64_t n, int32_t d, int32_t n_clusters, ui
     RBQ_CHECK(adist.alloc(sizeof(float) * n, s));
     {
       AssignWork w;  // without room for its scratch: the canonical tiles
-      const bool tc = assign_tc_applies(n, n_clusters) && w.alloc(n, d, n_clusters, s) == RABITQ_OK;
-      cudaGetLastError();
+      bool tc = assign_tc_applies(n, n_clusters);
+      if (tc && w.alloc(n, d, n_clusters, s) != RABITQ_OK) {
+        cudaGetLastError();
+        set_error("");
+        tc = false;
+      }
       if (tc) {
         RBQ_CHECK(assign_rows(ddata, X->centroids, X->centroids_t, n, n_clusters, d, w, X->assign,
                               adist.as<float>(), s));
@@ -271,7 +276,6 @@ int rabitq_build(const float* data, int64_t n, int32_t d, int32_t n_clusters, ui
     RBQ_CHECK(counting_sort(X->assign, n, n_clusters, X->perm, X->bucket_off, s));
     RBQ_CHECK(invert_perm(X->perm, n, X->inv_perm, s));
     RBQ_CHECK(gather_rows_f32(ddata, d, X->perm, n, d, X->data_b, s));
-    RBQ_CHECK(pack_rows(X, s));
     RBQ_CHECK(adist_b.alloc(sizeof(float) * n, s));
     RBQ_CHECK(gather_rows_f32(adist.as<float>(), 1, X->perm, n, 1, adist_b.as<float>(), s));
     RBQ_CHECK(sample_rotation_dev(seed, dpad, X->P64, X->P32, s));
@@ -280,6 +284,7 @@ int rabitq_build(const float* data, int64_t n, int32_t d, int32_t n_clusters, ui
                          X->ptc, dpad, n_clusters, dpad, d, s));
     RBQ_CHECK(encode_dev(X, adist_b.as<float>(), s));
     RBQ_CHECK(max_bucket_size(X, s));
+    RBQ_CHECK(pack_rows(X, s));
     RBQ_CUDA(cudaStreamSynchronize(s));
     return RABITQ_OK;
   };
@@ -897,8 +902,8 @@ int rabitq_index_load(const char* path, const rabitq_build_opts* opts, rabitq_in
       st = fail(RABITQ_ECUDA, "copy of P to the device failed");
     if (st == RABITQ_OK) st = pack_pt(X, nullptr);
   }
-  if (st == RABITQ_OK) st = pack_rows(X, nullptr);
   if (st == RABITQ_OK) st = max_bucket_size(X, nullptr);
+  if (st == RABITQ_OK) st = pack_rows(X, nullptr);
   if (st != RABITQ_OK) {
     free_index_arrays(X);
     delete X;

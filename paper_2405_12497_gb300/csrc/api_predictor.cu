@@ -46,6 +46,7 @@ int new_predictor(int32_t K, int32_t nprobe_max, rabitq_predictor** out) {
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&pr->params), sizeof(float) * kMlpParams);
   if (e == cudaSuccess) e = cudaMalloc(&pr->params_bf16, sizeof(uint16_t) * kMlpParams);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     free_predictor(pr);
     return fail(RABITQ_ENOMEM, std::string("predictor allocation failed: ") + cudaGetErrorString(e));
   }

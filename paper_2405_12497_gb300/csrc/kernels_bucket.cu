@@ -1554,10 +1554,15 @@ inline unsigned blocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
 
-// The 8-bit copy of the rows (after data_b is final). Without memory for it
-// the re-rank scores every row exactly.
+// The 8-bit copy of the rows (once everything else of the index is made).
+// Without memory for it the re-rank scores every row exactly; so that it never
+// costs a search or another index theirs, it is made only where a sixteenth of
+// the device's memory (18 GB) stays free beside it.
 int pack_rows(rabitq_index* X, cudaStream_t s) {
   const int64_t stride = row_stride(X->d);
+  size_t room = 0, total = 0;
+  RBQ_CUDA(cudaMemGetInfo(&room, &total));
+  if ((size_t)(X->n * stride) + total / 16 > room) return RABITQ_OK;
   if (cudaMalloc(reinterpret_cast<void**>(&X->rows8), (size_t)(X->n * stride)) != cudaSuccess) {
     cudaGetLastError();
     X->rows8 = nullptr;

@@ -561,6 +561,7 @@ int DevBuf::alloc(size_t bytes, cudaStream_t st) {
   cudaError_t e = cudaMallocAsync(&p, bytes, st);
   if (e != cudaSuccess) {
     p = nullptr;
+    cudaGetLastError();  // (the next launch's check must not find it)
     return fail(RABITQ_ENOMEM, std::string("device allocation failed: ") + cudaGetErrorString(e));
   }
   return RABITQ_OK;
@@ -709,8 +710,9 @@ int sample_rotation_dev(uint64_t seed, int32_t dpad, double* P64, float* P32, cu
   return RABITQ_OK;
 }
 
-int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters, int64_t sample,
-               uint64_t seed, float* centroids, cudaStream_t s) {
+namespace {
+int kmeans_run(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters, int64_t sample,
+               uint64_t seed, float* centroids, bool* tensor_cores, cudaStream_t s) {
   // training set: every point, or the Philox-sampled subset (ascending id)
   DevBuf train_buf, ids;
   const float* train = data;
@@ -748,9 +750,10 @@ int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters
   RBQ_CHECK(a.alloc(sizeof(int32_t) * m, s));
   RBQ_CHECK(perm.alloc(sizeof(int32_t) * m, s));
   RBQ_CHECK(off.alloc(sizeof(int32_t) * (K + 1), s));
-  AssignWork w;  // without room for its scratch: the canonical tiles
-  const bool tc = iters > 0 && assign_tc_applies(m, K) && w.alloc(m, d, K, s) == RABITQ_OK;
-  cudaGetLastError();
+  AssignWork w;
+  const bool tc = *tensor_cores && iters > 0 && assign_tc_applies(m, K);
+  *tensor_cores = tc;
+  if (tc) RBQ_CHECK(w.alloc(m, d, K, s));
   for (int it = 0; it < iters; ++it) {
     RBQ_CHECK(transpose_f32(centroids, K, d, ct.as<float>(), s));
     if (tc)
@@ -764,6 +767,20 @@ int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters
     RBQ_CUDA(cudaGetLastError());
   }
   return tc ? w.check(s) : RABITQ_OK;
+}
+}  // namespace
+
+// Assignment from tensor-core products where it applies; where its scratch (2
+// GiB at most) or anything beside it finds no memory, the canonical tiles.
+int kmeans_dev(const float* data, int64_t n, int32_t d, int32_t K, int32_t iters, int64_t sample,
+               uint64_t seed, float* centroids, cudaStream_t s) {
+  bool tc = true;
+  const int st = kmeans_run(data, n, d, K, iters, sample, seed, centroids, &tc, s);
+  if (st != RABITQ_ENOMEM || !tc) return st;
+  cudaGetLastError();
+  set_error("");
+  tc = false;
+  return kmeans_run(data, n, d, K, iters, sample, seed, centroids, &tc, s);
 }
 
 int encode_dev(rabitq_index* X, const float* adist_b, cudaStream_t s) {

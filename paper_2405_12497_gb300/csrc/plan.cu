@@ -193,6 +193,7 @@ int rabitq_plan_create(const rabitq_index* X, const rabitq_predictor* pr, int64_
     if (opts.collect_stats)
       for (auto& ev : P->ev)
         if (e == cudaSuccess) e = cudaEventCreate(&ev);
+    if (e != cudaSuccess) cudaGetLastError();
     if (e != cudaSuccess)
       st = fail(RABITQ_ENOMEM, std::string("rabitq_plan_create: ") + cudaGetErrorString(e));
   }

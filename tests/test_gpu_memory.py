@@ -86,3 +86,33 @@ for less in (20, 100, 180, 300, 1000):
 print("ok")
 """)
     assert "ok" in out
+
+
+# the assignment's tiles and lists take 1 GB here, the rows' 8-bit copy 0.4 GB:
+# a build that fits without them fits with any more memory, too
+def test_build_with_little_memory():
+    out = _run("""
+n, K = 4_000_000, 64
+data = torch.randn((n, 64), generator=g, device="cuda")
+want = R.Index.build(data, K, seed=2, kmeans_iters=2)
+cen, codes = want.centroids(), want.codes()
+want.free()
+fits = []
+for mb in range(1100, 3300, 100):
+    held = leave(mb * MB)
+    try:
+        G = R.Index.build(data, K, seed=2, kmeans_iters=2)
+    except R.RabitqError as e:
+        assert e.code == -2, e
+        fits.append(False)
+    else:
+        fits.append(True)
+        if len(fits) % 5 == 0:
+            assert (G.centroids() == cen).all() and (G.codes() == codes).all(), mb
+        G.free()
+    del held
+print("".join(".x"[f] for f in fits))
+assert fits[-1] and fits == sorted(fits), fits
+print("ok")
+""")
+    assert "ok" in out
