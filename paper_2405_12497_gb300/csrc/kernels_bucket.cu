@@ -617,7 +617,8 @@ __global__ void __launch_bounds__(kThreads) bucket_tau_kernel(const uint32_t* __
 // value with fewer than 20 roundings of magnitudes bounded by M = |F1| +
 // |add| + F2 (A sum(q_u) + |B| D') + F3 E + |tau|; the constants carry a
 // slack of 2^-18 of every term of M (c0, E', F1 and the threshold), more
-// than three times that error, so no pair the exact bound keeps is dropped.
+// than three times that error, and the threshold 1e-36 more for what underflows
+// (the smallest step is 1.4e-45), so no pair the exact bound keeps is dropped.
 // The few that pass are queued per lane (no votes, no cross-lane traffic)
 // and decided by the exact form, lane-parallel, when a queue fills and at
 // the end of the tile.
@@ -737,7 +738,7 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
         if (j >= padded) continue;
         const bool none = j >= x.cols;
         const float thr = none ? __int_as_float(0xff800000)
-                               : (tau[u] - m[u].w) + kGSlack * (fabsf(m[u].w) + fabsf(tau[u]));
+                               : (tau[u] - m[u].w) + (kGSlack * (fabsf(m[u].w) + fabsf(tau[u])) + 1e-36f);
         M.ex[j] = m[u];
         M.pt[j] = make_float2(ps[u], tau[u]);
         M.q[j] = q[u];

@@ -157,3 +157,18 @@ def test_learned_plans(R, nq, nprobe_max):
         assert torch.equal(ids, want[0])
         assert torch.equal(dist.view(torch.int32), want[1].view(torch.int32))
     assert torch.equal(plan.nprobe[:nq], npq)
+
+
+# squared distances down to FP32's smallest numbers
+@pytest.mark.parametrize("scale", [1e-18, 1e-20, 3e-21, 1e-22])
+def test_tiny_values(R, oracle_mod, scale):
+    rng = np.random.default_rng(5)
+    data = (_mix(rng, 20_000, 64) * scale).astype(np.float32)
+    Q = (_mix(rng, 2000, 64) * scale).astype(np.float32)
+    G = R.Index.build(data, 8, seed=2, kmeans_iters=2)
+    O = oracle_mod.OracleIndex(data, K=8, seed=2, iters=2)
+    for k, nprobe, eps0 in ((10, 4, 0.0), (10, 8, 0.5), (100, 8, 1.9)):
+        ids, dist = _check(R, G, Q, k, nprobe, eps0=eps0)
+        ids_o, dist_o = O.search(Q[:50], k, nprobe, eps0=eps0)
+        assert np.array_equal(ids[:50], ids_o)
+        assert np.array_equal(dist[:50].view(np.uint32), dist_o.view(np.uint32))
