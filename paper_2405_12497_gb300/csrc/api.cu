@@ -24,6 +24,14 @@ int fail(int code, const std::string& msg) {
   return code;
 }
 
+int flag_status(int flag, const char* over) {
+  if (flag == kErrWait)
+    return fail(RABITQ_ETIMEOUT, "a tensor-core wait expired (probe scores or query rotation)");
+  if (flag == kErrScanWait)
+    return fail(RABITQ_ETIMEOUT, "a tensor-core wait expired in the bucket-major scan");
+  return flag ? fail(RABITQ_EOVERFLOW, over) : RABITQ_OK;
+}
+
 int check_device(int device, const char* who) {
   int cur = 0;
   RBQ_CUDA(cudaGetDevice(&cur));

@@ -84,6 +84,12 @@ namespace rbq {
 // error plumbing (thread-local message)
 void set_error(const std::string& msg);
 int fail(int code, const std::string& msg);
+// The status of a search's device error flag: 0 none, 1 a candidate list
+// overflowed (the message: over), kErr* a tensor-core wait expired.
+constexpr int kErrWait = 2, kErrScanWait = 3;
+int flag_status(int flag, const char* over);
+constexpr const char* kListsOver =
+    "a query's candidate list exceeded max_candidates; raise max_candidates";
 // EINVAL (message names `who`) unless the calling thread's current device is
 // `device`, the device an index, predictor or plan lives on: its arrays are
 // device pointers of that GPU only.

@@ -596,7 +596,7 @@ int AssignWork::check(cudaStream_t s) {
   int h = 0;
   RBQ_CUDA(cudaMemcpyAsync(&h, redo.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   RBQ_CUDA(cudaStreamSynchronize(s));
-  if (h) return fail(RABITQ_ECUDA, "a tensor-core wait expired in the k-means assignment");
+  if (h) return fail(RABITQ_ETIMEOUT, "a tensor-core wait expired in the k-means assignment");
   return RABITQ_OK;
 }
 

@@ -989,7 +989,7 @@ __global__ void __launch_bounds__(kGThreads, 2) bucket_scan_kernel(BucketParams 
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (tid == 0 && s_fail) atomicExch(P.err, 2);
+  if (tid == 0 && s_fail) atomicExch(P.err, kErrScanWait);
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr),
                  "r"(2 * kGN));

@@ -2961,12 +2961,7 @@ int search_popc_run(const SearchArgs& a, bool* by_bucket_out, cudaStream_t s) {
     for (int i = 0; i < 4; ++i) a.stage_ms[i] = acc_ms[i];
     for (auto& e : ev) cudaEventDestroy(e);
   }
-  if (h_err == 2)
-    return fail(RABITQ_ETIMEOUT, "a tensor-core wait expired (probe scores or query rotation)");
-  if (h_err)
-    return fail(RABITQ_EOVERFLOW,
-                "a query's candidate list exceeded max_candidates; raise max_candidates");
-  return RABITQ_OK;
+  return flag_status(h_err, kListsOver);
 }
 
 }  // namespace
@@ -3082,8 +3077,7 @@ int fused_grid(const SearchArgs& a, int* grid_out) {
 }
 
 // Enqueue the search of a.nq queries (chunks of what fits) on stream s. The
-// error flag is the first int of the scratch (1 = candidate overflow,
-// 2 = tensor-core wait expired); the caller zeroes it before the first call
+// error flag is the first int of the scratch (flag_status); the caller zeroes it before the first call
 // and reads it after the stream has drained. grid: CTAs of the fused kernel
 // (0 = one per SM); cap: candidate capacity per CTA.
 int search_enqueue_carved(const SearchArgs& a, unsigned char* scratch, size_t scratch_bytes,
@@ -3291,11 +3285,7 @@ int search_dev_prealloc(const SearchArgs& a_in, unsigned char* scratch, size_t s
   RBQ_CUDA(cudaStreamSynchronize(s));
   if (h_err[1])
     return fail(RABITQ_EINVAL, "a query has a non-finite value (outputs undefined)");
-  if (h_err[0] == 2) return fail(RABITQ_ETIMEOUT, "a tensor-core wait expired (probe scores or query rotation)");
-  if (h_err[0])
-    return fail(RABITQ_EOVERFLOW,
-                "a query's candidate list exceeded the fixed scratch's capacity");
-  return RABITQ_OK;
+  return flag_status(h_err[0], "a query's candidate list exceeded the fixed scratch's capacity");
 }
 
 
