@@ -2,8 +2,8 @@
 
 Metric: QPS at recall@100 = 0.95 on one GB300 (plus the code-scan bandwidth
 against the HBM peak). Workload: 1M x 128 SIFT-shaped synthetic vectors,
-10k queries, IVF K = 4096, B_q = 4, eps0 = 1.9, k = 100, FP32 rotation,
-popcount scan. Two legs, each at mean recall@100 >= 0.95 against exact
+10k queries, IVF K = 4096, B_q = 4, eps0 = 1.9, k = 100, FP32 rotation, the
+scan that AUTO takes (config.scan). Two legs, each at mean recall@100 >= 0.95 against exact
 ground truth: fixed nprobe (swept; the smallest value reaching the target) and
 learned per-query nprobe (the MLP predictor trained on separately drawn
 queries, its multiplier raised until the target is met). The headline value is
@@ -235,10 +235,10 @@ def run_ours(args, rank, world):
                   "autotune": {"chosen": t_best, "candidates": t_all,
                                "tuned_on": "the calibration queries"}})
     fixed["roofline"] = roofline(G, qd, w, chosen, None, fixed["fused_ms"], hbm, src,
-                                 "fixed" + tag)
+                                 "fixed" + tag, fixed["tile"])
     fixed["scan_gbs"] = fixed["roofline"].pop("scan_gbs")
     fixed["ns_per_code"] = fixed["roofline"].pop("ns_per_code")
-    fixed["gpu_launches_per_step"] = 4
+    fixed["gpu_launches_per_step"] = launches_per_step(fixed["tile"], w, chosen)
     legs = {"fixed": fixed}
 
     # ---- leg 2: learned per-query nprobe
@@ -320,7 +320,9 @@ def run_ours(args, rank, world):
                    "operating_point": "nprobe / multiplier calibrated on 10k held-out "
                                       "calibration queries; recall measured on the "
                                       "evaluation queries",
-                   "rotation": "fp32", "scan": "popcount",
+                   "rotation": "fp32",
+                   "scan": "bucket-major products on the tensor cores"
+                           if by_bucket(best["tile"]) else "popcount, " + str(best["tile"]["layout"]),
                    "launch": "CUDA graph replay of the whole search (rabitq_plan_run)",
                    "l2": "flushed before each step",
                    "parallelism": f"replicas x{world} (every rank searches its own copy of "
@@ -335,7 +337,7 @@ def run_ours(args, rank, world):
                 "recall_at_100": round(e2e_rec, 4),
                 "path": "rabitq_plan_search: pinned host queries -> plan -> pinned host results"},
         "batch1_latency_us": latency,
-        "popc_roof": popc_roof(best, w, G),
+        "popc_roof": None if by_bucket(best["tile"]) else popc_roof(best, w, G),
         "gpu_launches": best["gpu_launches_per_step"] * args.steps,
         "clocks": fixed.pop("clocks"),
         "legs": legs,
@@ -446,7 +448,8 @@ def cold_scan_leg(args, G, qd, gt, w, flush, stream, dist, hbm, src):
                        max_candidates=1 << 18)
     leg = time_leg(args, plan, qd, gt, w, flush, stream, dist, name="cold_scan")
     leg.pop("_plan")
-    rl = roofline(G, qd, w, npb, None, leg["fused_ms"], hbm, src, f"cold{npb}")
+    tile = plan.tile()
+    rl = roofline(G, qd, w, npb, None, leg["fused_ms"], hbm, src, f"cold{npb}", tile)
     index_mb = G.n * (G.dpad / 8 + 16) / 1e6
     return {"nprobe": npb, "value": leg["value"], "unit": "queries/s",
             "recall_at_100": leg["recall_at_100"], "fused_ms": round(leg["fused_ms"], 4),
@@ -529,6 +532,23 @@ def batch1_latency(G, pa, qd, w, flush, n=200):
             "mode": "learned nprobe" if pa["predictor"] is not None else f"nprobe {pa['nprobe']}"}
 
 
+def by_bucket(tile) -> bool:
+    return tile["layout"] == "bucket-major"
+
+
+def launches_per_step(tile, w, nprobe, learned=False) -> int:
+    """Kernels of one graph replay (plans with stage times): query preparation
+    and probe scores, selection (with its redo launch where a warp takes a
+    query, and the learned counts' network and redo), rotation, then the scan:
+    ten bucket-major launches, or the per-query kernel (preceded by the work
+    order's two where counts differ)."""
+    select = 2 if w.nq >= 1024 and (learned or nprobe <= 64) else 1
+    if learned:
+        select += 1 + (1 if nprobe > 64 else 0)
+    scan = 10 if by_bucket(tile) else (3 if learned else 1)
+    return 2 + select + 1 + scan
+
+
 def popc_roof(best, w, G):
     """The popcount co-bound of the scan: B_q * D'/32 32-bit POPC per
     (query, code) at 16 POPC per clock per SM (sm_80+ rate) and the sampled
@@ -548,7 +568,7 @@ def popc_roof(best, w, G):
 def time_leg(args, plan, qd, gt, w, flush, stream, dist, clocks_on=False, name="leg"):
     """Time K graph replays of a plan (W warm-up replays first), L2 flushed
     before each; per-step device time by CUDA events on the launching stream,
-    the fused kernel's time by the event nodes inside the graph."""
+    the stages' times by the event nodes inside the graph."""
     import torch
     from paper_2405_12497_gb300 import rabitq  # noqa: F401
     plan.queries.copy_(qd)
@@ -623,26 +643,43 @@ def measured_traffic(workload: str, leg: str, nq: int):
     return int(ent["dram_bytes_per_query"] * nq)
 
 
-def roofline(G, qd, w, nprobe, per_query, fused_ms, hbm, src, leg):
-    """Algorithmic bytes of the fused scan/prune/re-rank kernel (one launch):
-    per estimated code D'/8 + 12 bytes, per survivor 4 D bytes -- counted on
-    the first 2000 queries by the trace and scaled to the batch."""
+def roofline(G, qd, w, nprobe, per_query, fused_ms, hbm, src, leg, tile):
+    """Algorithmic bytes of the scan/prune/re-rank stage against the HBM peak,
+    counted on the first 2000 queries by the trace and scaled to the batch.
+    Per-query kernel: per estimated code D'/8 + 12 bytes, per survivor 4 D.
+    Bucket-major: the codes and factors (D'/8 + 16) of the buckets that the
+    counted queries probe, once for the batch, and the survivors' rows, each
+    row of the data at most once; the stage is bound by the latency of its
+    steps, not by these bytes, so frac is small. scan_gbs counts the code bytes
+    once per (query, code) pair in both cases: an effective rate, which the
+    bucket-major scan may have above the peak."""
     n = min(2000, w.nq)
     t = G.search_trace(qd[:n], w.k, nprobe, bq=w.bq, eps0=w.eps0, max_candidates=1 << 20,
                        per_query_nprobe=None if per_query is None else per_query[:n])
     pairs_per_q = float(t["n_pairs"].double().mean())
     surv_per_q = float(t["n_surv"].double().mean())
+    probed = np.unique(t["probe_ids"].cpu().numpy())
     del t
-    bytes_launch = w.nq * (pairs_per_q * (G.dpad / 8 + 12) + surv_per_q * 4 * w.d)
-    achieved = bytes_launch / (fused_ms / 1e3) / 1e9
     scan_bytes = w.nq * pairs_per_q * (G.dpad / 8 + 12)
-    return {"kernel": "fused_search_kernel", "bound": "hbm", "achieved": round(achieved, 1),
-            "peak": hbm, "unit": "GB/s", "frac": round(achieved / hbm, 4),
-            "traffic": measured_traffic(w.name, leg, w.nq),
-            "peak_source": src, "algorithmic_bytes_per_launch": int(bytes_launch),
-            "pairs_per_query": round(pairs_per_q, 1), "survivors_per_query": round(surv_per_q, 1),
-            "scan_gbs": round(scan_bytes / (fused_ms / 1e3) / 1e9, 1),
-            "ns_per_code": round(fused_ms * 1e6 / (w.nq * pairs_per_q), 4)}
+    out = {"kernel": "fused_search_kernel", "bound": "hbm"}
+    if by_bucket(tile):
+        sizes = np.diff(G.buckets()[0])
+        codes = float(sizes[probed[probed >= 0]].sum())
+        bytes_launch = codes * (G.dpad / 8 + 16) + min(G.n, w.nq * surv_per_q) * 4 * w.d
+        out = {"kernel": "bucket_scan_kernel, bucket_tail_kernel", "bound": "latency",
+               "tensor_tflops": round(2 * 2 * w.nq * pairs_per_q * G.dpad / fused_ms / 1e9, 1),
+               "traffic": None}
+    else:
+        bytes_launch = scan_bytes + w.nq * surv_per_q * 4 * w.d
+        out["traffic"] = measured_traffic(w.name, leg, w.nq)
+    achieved = bytes_launch / (fused_ms / 1e3) / 1e9
+    out.update({"achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
+                "frac": round(achieved / hbm, 4), "peak_source": src,
+                "algorithmic_bytes_per_launch": int(bytes_launch),
+                "pairs_per_query": round(pairs_per_q, 1), "survivors_per_query": round(surv_per_q, 1),
+                "scan_gbs": round(scan_bytes / (fused_ms / 1e3) / 1e9, 1),
+                "ns_per_code": round(fused_ms * 1e6 / (w.nq * pairs_per_q), 4)})
+    return out
 
 
 def learned_leg(args, G, qd, gt, w, fixed_nprobe, flush, stream, dist, hbm, src, cqd, cgt):
@@ -675,10 +712,10 @@ def learned_leg(args, G, qd, gt, w, fixed_nprobe, flush, stream, dist, hbm, src,
     plan = rabitq.Plan(G, w.k, 0, w.nq, bq=w.bq, eps0=w.eps0, predictor=pr, stats=True)
     leg = time_leg(args, plan, qd, gt, w, flush, stream, dist, name="learned")
     leg["roofline"] = roofline(G, qd, w, args.nprobe_max, npq, leg["fused_ms"], hbm, src,
-                               "learned")
+                               "learned", plan.tile())
     leg["scan_gbs"] = leg["roofline"].pop("scan_gbs")
     leg["ns_per_code"] = leg["roofline"].pop("ns_per_code")
-    leg["gpu_launches_per_step"] = 12
+    leg["gpu_launches_per_step"] = launches_per_step(plan.tile(), w, args.nprobe_max, True)
     leg["_pred_obj"] = pr
     npf = npq.double().cpu().numpy()
     leg.update({
@@ -905,7 +942,7 @@ def deep_legs(args, flush, stream, dist, hbm, src):
                                                    for a, b in sorted(sweep.items())},
                   "autotune": {"chosen": t_best, "candidates": t_all}})
     fixed["roofline"] = roofline(G, qd, w, chosen, None, fixed["fused_ms"], hbm, src,
-                                 "deep_fixed")
+                                 "deep_fixed", fixed["tile"])
     f_ids, f_dist = fixed.pop("_ids"), fixed.pop("_dist")
     fixed.pop("_npq")
     fixed.pop("_plan")
@@ -928,7 +965,7 @@ def deep_legs(args, flush, stream, dist, hbm, src):
                         max_candidates=cap)
     learned = time_leg(args, lplan, qd, gt, w, flush, stream, dist, name="deep_learned")
     learned["roofline"] = roofline(G, qd, w, 256, npq, learned["fused_ms"], hbm, src,
-                                   "deep_learned")
+                                   "deep_learned", lplan.tile())
     l_ids, l_dist, l_npq = learned.pop("_ids"), learned.pop("_dist"), learned.pop("_npq")
     learned.pop("_plan")
     l_tile = lplan.tile()
@@ -952,7 +989,8 @@ def deep_legs(args, flush, stream, dist, hbm, src):
     cold["nprobe"] = 128
     cold["tile"] = cplan.tile()
     cplan.free()
-    cold["roofline"] = roofline(G, qd, w, 128, None, cold["fused_ms"], hbm, src, "deep_cold128")
+    cold["roofline"] = roofline(G, qd, w, 128, None, cold["fused_ms"], hbm, src, "deep_cold128",
+                                cold["tile"])
     cold["codes_and_factors_mb"] = round(G.n * (G.dpad / 8 + 16) / 1e6, 1)
     out = {"workload": w.name + f"-sigma{DEEP_SIGMA}", "n": w.n, "d": w.d,
            "n_clusters": w.n_clusters, "k": w.k, "bq": w.bq, "eps0": w.eps0,
