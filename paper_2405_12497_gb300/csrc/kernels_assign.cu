@@ -7,7 +7,7 @@
 // by its own, the centroids by one) so that the largest magnitude lies in
 // [2^13, 2^14), and rounded to FP16: the same 11 significant bits as TF32 at
 // twice its rate and half its bytes. What falls under FP16's smallest normal
-// is off by at most 2^-39 of the largest element, far inside the bound's 5%.
+// is off by at most 2^-38 of the largest element, far inside the bound's 5%.
 // The products <x, c>~ give s_c = ||c||^2 - 2 <x, c>~, which differs from the
 // canonical score less ||x||^2 (the same for every c) by at most eps_c
 // (ProbeEps: operand rounding, accumulation, the canonical fold's own error,
