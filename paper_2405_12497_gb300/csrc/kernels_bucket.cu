@@ -33,15 +33,17 @@
 // them redone, 4.66 all per query, 3.68 so).
 //
 // Measured (GB300, order to re-rank of one batch, per-query kernel -> this):
-//   10k queries x 62 probes, 1M x 128, K 4096, k 100        4.83 -> 2.47 ms
+//   10k queries x 62 probes, 1M x 128, K 4096, k 100        4.83 -> 2.30 ms
 //   10k queries x 128 probes, 2M x 256, K 4096, k 100      17.5  -> 6.44 ms
 //   4000 queries x 16 probes, 1M x 128, K 4096, k 10        0.57 -> 0.37 ms
 //   1000 queries x 32 probes, 200k x 960, K 1024, k 100     1.27 -> 0.95 ms
-// Of the first: quantization 0.21, tau0 0.12, passes 0.42 and 0.73, tail 0.95.
-// The passes are bound by the epilogue's issue slots (some 25 instructions per
-// column of 32 codes) and, in pass 2, by the latency of the hits' list slots;
-// the tensor cores are about a tenth busy. The tail is bound by the latency of
-// its short steps.
+// Of the first: quantization 0.22, tau0 0.13, passes 0.43 and 0.71, tail 0.86.
+// The quantization keeps 74% of the issue slots busy. The passes keep half of
+// them busy and the tensor pipe 5 and 3%, DRAM below 10%: they wait for the
+// hits' list slots and the items' constants (most stalls are on global loads and
+// atomics), and their time hardly follows their work (8000 learned queries:
+// 0.17 ms for pass 2 with all pairs or a quarter less). The tail is bound by the
+// latency of its short steps (loads, then barriers; DRAM 36%).
 #include <algorithm>
 #include <cstring>
 
