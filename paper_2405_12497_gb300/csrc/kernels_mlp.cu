@@ -135,18 +135,24 @@ __device__ __forceinline__ int probe_count(float y, float mult, int nmax) {
 
 // Fused inference: kQB queries per block, four hidden units x four queries
 // per thread (units 4 ug .. 4 ug + 3 of query group qg), accumulated in pairs
-// of units by packed FMAs. The activations are stored transposed
+// of queries by packed FMAs. The activations are stored transposed
 // ([unit][query]): each step of a dot product reads the four queries of one
-// unit with one 16-byte broadcast load and the four weights with one 8-byte
-// load, for 16 FMAs; the next eight steps' weights are on their way while
-// eight are used. (One unit x 32 queries per thread read eight times as much
-// shared memory per FMA: 80 us per 8000 queries, this form 44. Scalar FMAs
-// instead of packed ones 48 us, 8 x 4 tiles 50, 8 x 8 tiles 54: fewer warps.)
+// unit with one 16-byte broadcast load, already in pairs, and the four weights
+// with one 8-byte load, for 16 FMAs. The weights pass through shared memory, 32
+// rows a stage, the next stage on its way (cp.async) while one is used: the four
+// warps that want the same ones fetch them once. 46 us per 8000 queries, and a
+// learned plan that selects in two parts (search_enqueue_carved) 1.3% faster than
+// with weights from L2 to registers eight rows ahead (47 us). Alone all forms take
+// about that: pairs of units 47, 32 queries per block 46 (but a request of 53
+// queries 179 us instead of 171), scalar FMAs 48, one unit x 32 queries per thread
+// 80; no counter is near its limit (FMA pipe 42%, issue slots 30%).
 // With out_ids the block also writes its queries' probe lists: the first
 // probe count entries of the navail selected ones (rows of navail in, of ldo
 // out); a query that needs more goes to redo (count, then the queries).
 constexpr int kQB = 16, kInferThreads = 256;
-constexpr size_t kInferSmem = sizeof(float) * (kQB * kF + 2 * kQB * kH + kH);
+constexpr int kInferRows = 32;  // weight rows per stage
+constexpr int kInferStage = kInferRows * kH * 2;
+constexpr size_t kInferSmem = sizeof(float) * (kQB * kF + 2 * kQB * kH + kH) + 2 * kInferStage;
 
 __device__ __forceinline__ uint64_t pack2f(float a, float b) {
   uint64_t r;
@@ -159,12 +165,8 @@ __device__ __forceinline__ void unpack2f(uint64_t v, float& a, float& b) {
 __device__ __forceinline__ void fma2f(uint64_t& c, uint64_t a, uint64_t b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
 }
-// two packed BF16 values as a pair of FP32
-__device__ __forceinline__ uint64_t bf2_pair(uint32_t w) {
-  return pack2f(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
 
-__global__ void __launch_bounds__(kInferThreads, 4) mlp_infer_kernel(
+__global__ void __launch_bounds__(kInferThreads, 3) mlp_infer_kernel(
     const float* __restrict__ sel_dist, int64_t ld, int64_t nq, int navail, float s0,
     const __nv_bfloat16* __restrict__ P, float mult, int nmax, float* __restrict__ feat_out,
     float* __restrict__ y_out, int32_t* __restrict__ np_out, MlpLists L) {
@@ -196,56 +198,68 @@ __global__ void __launch_bounds__(kInferThreads, 4) mlp_infer_kernel(
   __syncthreads();
   // a warp: 32 unit groups of one half of the units, one query group
   const int qg = (tid >> 5) & 3, ug = ((tid >> 7) << 5) + (tid & 31);
-  uint64_t acc[2][4];  // [unit pair][query]
+  uint64_t acc[4][2];  // [unit][query pair]
   // one dense layer: acc = fold_j fma(in[j][q], W[j][n], acc), ascending j
+  char* wst = reinterpret_cast<char*>(w3 + kH);  // two stages of weights
   auto layer = [&](const float* inT, int nin, int woff) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[u][q] = 0ull;
-    const uint2* w2 = reinterpret_cast<const uint2*>(P + woff) + ug;
-    const float4* a4 = reinterpret_cast<const float4*>(inT) + qg;
-    uint2 wn[8];
+      for (int q = 0; q < 2; ++q) acc[u][q] = 0ull;
+    const char* src = reinterpret_cast<const char*>(P + woff);
+    auto fetch = [&](int st) {
+      const uint32_t dst = (uint32_t)__cvta_generic_to_shared(wst + (st & 1) * kInferStage);
 #pragma unroll
-    for (int r = 0; r < 8; ++r) wn[r] = __ldg(w2 + r * (kH / 4));
-    for (int j0 = 0; j0 < nin; j0 += 8) {
-      uint2 wc[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) wc[r] = wn[r];
-      const int jn = j0 + 8 < nin ? j0 + 8 : j0;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) wn[r] = __ldg(w2 + (jn + r) * (kH / 4));
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const float4 a = a4[(j0 + r) * (kQB / 4)];
-        const uint64_t wp[2] = {bf2_pair(wc[r].x), bf2_pair(wc[r].y)};
-        const uint64_t ap[4] = {pack2f(a.x, a.x), pack2f(a.y, a.y), pack2f(a.z, a.z),
-                                pack2f(a.w, a.w)};
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) fma2f(acc[u][q], ap[q], wp[u]);
+      for (int o = 16 * tid; o < kInferStage; o += 16 * kInferThreads)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + o),
+                     "l"(src + st * kInferStage + o)
+                     : "memory");
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const ulonglong2* a4 = reinterpret_cast<const ulonglong2*>(inT) + qg;
+    const int ns = nin / kInferRows;
+    fetch(0);
+    for (int st = 0; st < ns; ++st) {
+      if (st + 1 < ns) {
+        fetch(st + 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
       }
+      __syncthreads();
+      const uint2* w2 = reinterpret_cast<const uint2*>(wst + (st & 1) * kInferStage) + ug;
+#pragma unroll 8
+      for (int r = 0; r < kInferRows; ++r) {
+        const int j = st * kInferRows + r;
+        const ulonglong2 a = a4[j * (kQB / 4)];
+        const uint2 wv = w2[r * (kH / 4)];
+        const uint32_t ws[2] = {wv.x, wv.y};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float w = __uint_as_float((u & 1) ? ws[u >> 1] & 0xffff0000u : ws[u >> 1] << 16);
+          const uint64_t ww = pack2f(w, w);
+          fma2f(acc[u][0], a.x, ww);
+          fma2f(acc[u][1], a.y, ww);
+        }
+      }
+      __syncthreads();
     }
   };
   auto bias_relu_store = [&](int boff, float* outT) {
     const uint2 bw = __ldg(reinterpret_cast<const uint2*>(P + boff) + ug);
-    const uint32_t bb[2] = {bw.x, bw.y};
+    const uint32_t bb[4] = {bw.x << 16, bw.x & 0xffff0000u, bw.y << 16, bw.y & 0xffff0000u};
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const float b0 = __uint_as_float(bb[u] << 16), b1 = __uint_as_float(bb[u] & 0xffff0000u);
-      float z0[4], z1[4];
+    for (int u = 0; u < 4; ++u) {
+      float z[4];
+      unpack2f(acc[u][0], z[0], z[1]);
+      unpack2f(acc[u][1], z[2], z[3]);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        unpack2f(acc[u][q], z0[q], z1[q]);
-        z0[q] = __fadd_rn(z0[q], b0);
-        z1[q] = __fadd_rn(z1[q], b1);
-        z0[q] = z0[q] > 0.0f ? z0[q] : 0.0f;
-        z1[q] = z1[q] > 0.0f ? z1[q] : 0.0f;
+        z[q] = __fadd_rn(z[q], __uint_as_float(bb[u]));
+        z[q] = z[q] > 0.0f ? z[q] : 0.0f;
       }
-      float4* o4 = reinterpret_cast<float4*>(outT + (4 * ug + 2 * u) * kQB) + qg;
-      o4[0] = make_float4(z0[0], z0[1], z0[2], z0[3]);
-      o4[kQB / 4] = make_float4(z1[0], z1[1], z1[2], z1[3]);
+      reinterpret_cast<float4*>(outT + (4 * ug + u) * kQB)[qg] =
+          make_float4(z[0], z[1], z[2], z[3]);
     }
   };
   layer(xT, kF, oW1);
