@@ -314,13 +314,16 @@ __device__ __forceinline__ double gs_fold(const double* __restrict__ f,
   return s;
 }
 
+// WHOLE: dpad is a multiple of 32, as in every index (the bound on o, which other
+// sizes need, makes 1024 rows 1% slower).
+template <bool WHOLE>
 __global__ void __launch_bounds__(kGsThreads, 1) gram_schmidt_kernel(
     const double* __restrict__ G, int dpad, double* P, double* PT, double* v, double* c,
     unsigned* bar, int* err) {
   extern __shared__ __align__(16) double gs_row[];  // the staged v or c
   __shared__ double s_norm;
   const int o = blockIdx.x * 32 + threadIdx.x;  // the lane's row and column
-  const bool lane = threadIdx.x < 32 && o < dpad;
+  const bool lane = threadIdx.x < 32 && (WHOLE || o < dpad);
   unsigned done = 0;
   double x[kGsAhead];
   auto meet = [&]() { return gs_barrier(bar, done += gridDim.x, err); };
@@ -699,7 +702,8 @@ int sample_rotation_dev(uint64_t seed, int32_t dpad, double* P64, float* P32, cu
   RBQ_CUDA(cudaMemsetAsync(bar, 0, 16, s));
   void* args[] = {&g, &dpad, &P64, &pt, &vp, &c, &bar, &err};
   // at most 128 CTAs (dpad <= 4096, any even size)
-  RBQ_CUDA(cudaLaunchCooperativeKernel((const void*)gram_schmidt_kernel, dim3((dpad + 31) / 32),
+  const auto fn = dpad % 32 ? gram_schmidt_kernel<false> : gram_schmidt_kernel<true>;
+  RBQ_CUDA(cudaLaunchCooperativeKernel((const void*)fn, dim3((dpad + 31) / 32),
                                        dim3(kGsThreads), args, sizeof(double) * dpad, s));
   to_f32_kernel<<<blocks_for(total, 256), 256, 0, s>>>(P64, total, P32);
   RBQ_CUDA(cudaGetLastError());
