@@ -1589,7 +1589,9 @@ bool bucket_applies(const SearchArgs& a, int64_t nq) {
   // Of the 500 points with 1000 queries and more, this rule leaves 12 with over
   // 3% and at most 10% against the per-query scan (four pairs alone: 80, up to
   // 59%: 1000 queries x 4 probes, 100k x 96, k = 100: 0.174 ms per query, 0.262
-  // so). Below a thousand queries the tail's last wave is mostly idle.
+  // so). The limit of a thousand queries is older than the one on the codes: below
+  // it 121 of 260 points are slower (the tail's last wave is mostly idle), but of
+  // the 93 that the latter admits only 3 (at most 16%), so it could come down.
   const double pairs = (double)nq * a.mean_probes;
   if (nq < 1000 || pairs < 4.0 * a.X->K) return false;
   const double work = pairs * a.X->n / a.X->K * a.X->dpad / 128.0;
